@@ -9,10 +9,11 @@
 // acts on every channel alike and the bias only on the value channel, which is
 // how value, Jacobian and Laplacian propagate through Eqs. (17)-(19), (24).
 //
-// Tiling: BM x BN output tile per CTA, BK-deep k-slices double-buffered in
+// FP32 tiling: BM x BN output tile per CTA, BK-deep k-slices double-buffered in
 // shared memory (transposed, padded, 16-byte vector accesses), TM x TN
 // register tile per thread split in two halves so that shared-memory reads
-// are conflict-free.
+// are conflict-free.  FP64 has a kernel of its own (gemm_nt_f64_kernel), whose
+// tile is chosen by the size.
 #include "common.cuh"
 
 namespace dq {
@@ -24,11 +25,6 @@ template <>
 struct Vec<float> {
   using type = float4;
   static constexpr int n = 4;
-};
-template <>
-struct Vec<double> {
-  using type = double2;
-  static constexpr int n = 2;
 };
 
 __device__ __forceinline__ int64_t row_offset(const RowMap& m, int64_t r) {
@@ -180,9 +176,129 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// FP64.  What bounds it is the FP64 pipe of the busiest SM (1.7 multiply-adds per clock and SM,
+// a warp instruction every 19 clocks: one CTA of eight warps keeps it full and shared-memory
+// traffic does not count), so what matters is that the multiply-adds, those of the padding
+// included, are spread evenly over the SMs; see the choice of the tile below.  A 64-row tile
+// leaves 120 of 152 SMs idle at the 2048 rows of a 512-walker LiH forward: with 64 x 64 tiles
+// only, the update map (K = 96, 32 outputs) took 107 us a launch and ten sampling sweeps 8.06 ms;
+// with the tile by size they take 3.34 ms.
+// k runs in order for every output, whatever the tile: all tiles give the same bits.
+constexpr int F64_BK = 32;
+
+template <int BM, int BN>
+__global__ void __launch_bounds__(256)
+    gemm_nt_f64_kernel(const double* __restrict__ X, RowMap mx, const double* __restrict__ W,
+                       const double* __restrict__ bias, int bias_period, double* __restrict__ Y, RowMap my, int64_t rows,
+                       int n_out, int K, int accumulate) {
+  constexpr int NT = 256;
+  constexpr int CT = BN < 16 ? BN : 16;  // threads along the columns
+  constexpr int TM = BM * CT / NT, TN = BN / CT;
+  static_assert(TM >= 1 && TM * (NT / CT) == BM && TN * CT == BN, "tile/thread mismatch");
+  constexpr int LA = BM * F64_BK / NT, LB = BN * F64_BK / NT;
+  __shared__ double As[F64_BK][BM + 1];
+  __shared__ double Bs[F64_BK][BN + 1];
+  const int tid = threadIdx.x, kk0 = tid % F64_BK, lr0 = tid / F64_BK;  // this thread loads column kk0 of rows lr0 + 8 i
+  const int tx = tid % CT, ty = tid / CT;
+  const int64_t row0 = (int64_t)blockIdx.x * BM;
+  const int col0 = blockIdx.y * BN;
+
+  const double* a_ptr[LA];
+  const double* b_ptr[LB];
+#pragma unroll
+  for (int i = 0; i < LA; ++i) {
+    const int64_t r = row0 + lr0 + i * (NT / F64_BK);
+    a_ptr[i] = r < rows ? X + row_offset(mx, r) + kk0 : nullptr;
+  }
+#pragma unroll
+  for (int i = 0; i < LB; ++i) {
+    const int n = col0 + lr0 + i * (NT / F64_BK);
+    b_ptr[i] = n < n_out ? W + (int64_t)n * K + kk0 : nullptr;
+  }
+  double ra[LA], rb[LB];
+  auto load = [&](int k0) {
+    const bool in = k0 + kk0 < K;
+#pragma unroll
+    for (int i = 0; i < LA; ++i) ra[i] = in && a_ptr[i] ? a_ptr[i][k0] : 0.0;
+#pragma unroll
+    for (int i = 0; i < LB; ++i) rb[i] = in && b_ptr[i] ? __ldg(b_ptr[i] + k0) : 0.0;
+  };
+  double acc[TM][TN] = {};
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += F64_BK) {
+    __syncthreads();  // the previous slice is consumed
+#pragma unroll
+    for (int i = 0; i < LA; ++i) As[kk0][lr0 + i * (NT / F64_BK)] = ra[i];
+#pragma unroll
+    for (int i = 0; i < LB; ++i) Bs[kk0][lr0 + i * (NT / F64_BK)] = rb[i];
+    __syncthreads();
+    if (k0 + F64_BK < K) load(k0 + F64_BK);
+    const int kn = min(F64_BK, K - k0);  // a multiple of 8
+#pragma unroll 8
+    for (int kk = 0; kk < kn; ++kk) {
+      double a[TM], b[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * (NT / CT)];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + j * CT];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int64_t r = row0 + ty + i * (NT / CT);
+    if (r >= rows) continue;
+    double* y = Y + row_offset(my, r);
+    const bool add_bias = bias != nullptr && (r % bias_period) == 0;
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int n = col0 + tx + j * CT;
+      if (n >= n_out) continue;
+      double v = acc[i][j];
+      if (add_bias) v += bias[n];
+      if (accumulate) v += y[n];
+      y[n] = v;
+    }
+  }
+}
+
 }  // namespace
 
 namespace {
+// The FP64 tile: the one that gives the busiest SM the fewest multiply-adds (its share of the
+// tiles, rounded up, times the tile's area, padding included); the larger tile where two agree.
+cudaError_t gemm_f64_dispatch(const double* X, RowMap mx, const double* W, const double* bias, int bias_period,
+                              double* Y, RowMap my, int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  using Kern = void (*)(const double*, RowMap, const double*, const double*, int, double*, RowMap, int64_t, int, int,
+                        int);
+  struct Tile {
+    int bm, bn;
+    Kern kern;
+  };
+  const Tile tiles[] = {{64, 64, gemm_nt_f64_kernel<64, 64>}, {64, 32, gemm_nt_f64_kernel<64, 32>},
+                        {32, 32, gemm_nt_f64_kernel<32, 32>}, {32, 16, gemm_nt_f64_kernel<32, 16>},
+                        {16, 16, gemm_nt_f64_kernel<16, 16>}};
+  const Tile* best = nullptr;
+  int64_t least = 0;
+  for (const Tile& t : tiles) {
+    const int64_t n = ((rows + t.bm - 1) / t.bm) * ((n_out + t.bn - 1) / t.bn);
+    const int64_t cost = (n + sms - 1) / sms * t.bm * t.bn;
+    if (best == nullptr || cost < least) {
+      best = &t;
+      least = cost;
+    }
+  }
+  const dim3 grid((unsigned)((rows + best->bm - 1) / best->bm), (unsigned)((n_out + best->bn - 1) / best->bn));
+  best->kern<<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate ? 1 : 0);
+  return cudaGetLastError();
+}
+
 template <class T, int BM, int BN, int BK>
 cudaError_t gemm_dispatch(const T* X, RowMap mx, const T* W, const T* bias, int bias_period, T* Y, RowMap my,
                           int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s) {
@@ -211,7 +327,7 @@ cudaError_t gemm_nt(const T* X, RowMap mx, const T* W, const T* bias, int bias_p
   if constexpr (sizeof(T) == 4) {
     return gemm_dispatch<T, 128, 128, 8>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate, s);
   } else {
-    return gemm_dispatch<T, 64, 64, 8>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate, s);
+    return gemm_f64_dispatch(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate, s);
   }
 }
 
