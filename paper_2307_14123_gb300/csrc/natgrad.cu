@@ -7,12 +7,13 @@
 // (gemm_tc.cu), the system is solved by conjugate gradients preconditioned with
 // its diagonal (walkers' gradient norms span orders of magnitude near the
 // nodes), in FP64 with fixed-order reductions (deterministic), and delta =
-// Gc^T x is a weighted column sum.  The conjugate-gradient loop runs as a fixed sequence of launches
-// that stop working once a flag in device memory says the residual is small
-// enough, so the whole call can be captured in a CUDA graph.
+// Gc^T x is a weighted column sum.  The conjugate gradients run in one cooperative kernel whose
+// CTAs meet at one grid barrier per iteration and leave the loop when the residual is small
+// enough, so the call needs no host synchronisation and can be captured in a CUDA graph.
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace dq {
 namespace {
@@ -216,6 +217,162 @@ __global__ void ng_cg_direction_kernel(int64_t B, const double* __restrict__ z, 
     p[i] = z[i] + beta * p[i];
 }
 
+// ---------------------------------------------------------------------------
+// All iterations in one cooperative kernel (ng_cg_init_kernel sets the system up).
+// What bounds an iteration: the matvec's B^2 FP64 multiply-adds (1.7 per clock
+// and SM: 2 us at B = 1024, 33 us at 4096) and the trips to the other SMs, not
+// memory (T stays in L2, or in L1 up to B of about 1200).  So every CTA owns rpc
+// rows of T, and keeps p, r and 1 / diag of the whole system in shared memory:
+// it publishes its rows of A p, meets the others at one grid barrier, and then
+// forms pAp, r, rr, rz and the next p of all walkers by itself, as every other
+// CTA does.  That spends 6 B redundant multiply-adds per CTA instead of a second
+// barrier with its reduction, and every CTA takes the same decisions from the
+// same bits.  The sums are added in the order of the kernels above, which serve
+// the systems that do not fit here: both give the same bits.
+// Against those (three launches per iteration, always max_iter of them; 17.4 +
+// 9.9 + 3.1 us each at B = 1024 until the residual is small) the call on 1024
+// walkers x 412,656 parameters takes 15.2 ms instead of 17.7, and a LiH training
+// step of 1024 walkers 8.0 ms instead of 10.7.
+// The barrier's wait is bounded; on a timeout every CTA leaves and
+// DQ_FLAG_TIMEOUT is set.
+// ---------------------------------------------------------------------------
+constexpr int kCgThreads = 512;
+constexpr int kCgWarps = kCgThreads / 32;
+constexpr int kCgMaxGroups = 64;                  // groups of kNgThreads walkers: B <= 16384
+constexpr size_t kCgMaxSmem = 227 * 1024 - 4096;  // 4 KB left for the static arrays
+
+inline size_t ng_solve_smem(int64_t B) { return (size_t)3 * B * sizeof(double); }
+
+// ng_block_sum's tree over kNgThreads = 256 values by one warp, lane l holding the values
+// l + 32 m in v[m]; every lane returns the sum.
+__device__ __forceinline__ double cg_tree256(double (&v)[8]) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) v[m] += v[m + 4];
+  v[0] += v[2];
+  v[1] += v[3];
+  double s = v[0] + v[1];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+// The same over n <= 256 values of shared memory (zeros after them).
+__device__ __forceinline__ double cg_tree256(const double* a, int n, int lane) {
+  double v[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) v[m] = lane + 32 * m < n ? a[lane + 32 * m] : 0.0;
+  return cg_tree256(v);
+}
+
+__global__ void __launch_bounds__(kCgThreads, 1)
+    ng_cg_solve_kernel(const double* __restrict__ T, int B, int rpc, const double* __restrict__ r_in,
+                       const double* __restrict__ p_in, const double* __restrict__ dinv_in, double* Ap,
+                       double* __restrict__ x, CgScalars* sc, unsigned int* arrivals, unsigned int* status) {
+  extern __shared__ __align__(16) unsigned char cg_smem[];
+  double* p = reinterpret_cast<double*>(cg_smem);  // [B] direction
+  double* r = p + B;                               // [B] residual
+  double* dinv = r + B;                            // [B] 1 / diagonal
+  __shared__ double s_pap[kNgThreads], s_rr[kCgMaxGroups], s_rz[kCgMaxGroups];
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+  const int row0 = blockIdx.x * rpc, row1 = min(B, row0 + rpc);
+  const int n_oct = (B + kNgRowWarps - 1) / kNgRowWarps;  // groups of eight rows (ng_cg_matvec_kernel's CTAs)
+  const int n_grp = (B + kNgThreads - 1) / kNgThreads;    // groups of 256 walkers (ng_cg_update_kernel's CTAs)
+  static_assert(kNgRowWarps == 8 && kNgThreads == 256, "cg_tree256 and the octet sums follow these sizes");
+  for (int i = tid; i < B; i += kCgThreads) {
+    r[i] = r_in[i];
+    p[i] = p_in[i];
+    dinv[i] = dinv_in[i];
+  }
+  const double lam = sc->lam, tol2 = sc->tol2;
+  const int max_iter = sc->max_iter;
+  double rr = sc->rr, rz = sc->rz;
+  bool done = sc->done != 0;
+  double xi = 0;  // x of walker row0 + tid (tid < row1 - row0)
+  int it = 0;
+  __syncthreads();
+  for (; !done; ++it) {
+    double* Ab = Ap + (size_t)(it & 1) * B;  // two buffers: a CTA may still read the last iteration's
+    for (int i = row0 + warp; i < row1; i += kCgWarps) {
+      const double* Ti = T + (int64_t)i * B;
+      double s = 0;
+#pragma unroll 8
+      for (int j = lane; j < B; j += 32) s = fma(Ti[j], p[j], s);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) __stcg(Ab + i, fma(lam, p[i], s / (double)B));
+    }
+    __syncthreads();
+    if (tid == 0) {  // grid barrier: all rows of A p published
+      __threadfence();
+      atomicAdd(arrivals, 1u);
+      const unsigned int target = (unsigned int)(it + 1) * gridDim.x;
+      const long long t0 = clock64();
+      int ok = 1;
+      while ((int)(*(volatile unsigned int*)arrivals - target) < 0)
+        if (clock64() - t0 > tcp::kWaitCycles) {
+          ok = 0;
+          break;
+        }
+      __threadfence();
+      s_ok = ok;
+    }
+    __syncthreads();
+    if (!s_ok) {
+      if (tid == 0) atomicOr(status, (unsigned)DQ_FLAG_TIMEOUT);
+      break;
+    }
+    if (tid < kNgThreads) {  // p . A p: octets of rows, strided over 256 threads, then the tree
+      double s = 0;
+      for (int c = tid; c < n_oct; c += kNgThreads) {
+        double t[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int i = c * 8 + q;
+          t[q] = i < B ? __ldcg(Ab + i) * p[i] : 0.0;
+        }
+        s += ((t[0] + t[4]) + (t[2] + t[6])) + ((t[1] + t[5]) + (t[3] + t[7]));
+      }
+      s_pap[tid] = s;
+    }
+    __syncthreads();
+    const double pAp = cg_tree256(s_pap, kNgThreads, lane);
+    const double alpha = pAp > 0 ? rz / pAp : 0.0;
+    if (tid < row1 - row0) xi = fma(alpha, p[row0 + tid], xi);
+    for (int g = warp; g < n_grp; g += kCgWarps) {  // r -= alpha A p; the group's r.r and r.z
+      double vr[8], vz[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int i = g * kNgThreads + lane + 32 * m;
+        vr[m] = vz[m] = 0;
+        if (i < B) {
+          const double ri = fma(-alpha, __ldcg(Ab + i), r[i]);
+          r[i] = ri;
+          vr[m] = ri * ri;
+          vz[m] = ri * (ri * dinv[i]);
+        }
+      }
+      const double a = cg_tree256(vr), b = cg_tree256(vz);
+      if (lane == 0) {
+        s_rr[g] = a;
+        s_rz[g] = b;
+      }
+    }
+    __syncthreads();
+    rr = cg_tree256(s_rr, n_grp, lane);
+    const double rz_new = cg_tree256(s_rz, n_grp, lane);
+    const double beta = rz > 0 ? rz_new / rz : 0.0;
+    rz = rz_new;
+    done = rr <= tol2 || it + 1 >= max_iter || !(pAp > 0);
+    for (int i = tid; i < B; i += kCgThreads) p[i] = fma(beta, p[i], r[i] * dinv[i]);
+    __syncthreads();
+  }
+  if (tid < row1 - row0) x[row0 + tid] = xi;
+  if (blockIdx.x == 0 && tid == 0) {
+    sc->rr = rr;
+    sc->iter = it;
+  }
+}
+
 // delta[p] = sum_b x_b Gc[b][p] (fixed order over b); stats
 __global__ void ng_apply_kernel(const float* __restrict__ Gc, int64_t B, int64_t P, int64_t Pp,
                                 const double* __restrict__ x, float* __restrict__ delta) {
@@ -236,6 +393,31 @@ __global__ void ng_stats_kernel(const CgScalars* sc, double* stats) {
 inline unsigned ng_blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 inline size_t ng_align(size_t x) { return (x + 255) / 256 * 256; }
 
+// Launches the one-kernel iteration; false where it does not serve the system (its vectors exceed
+// shared memory, or the device cannot hold the grid at once), *e: a launch error.
+bool ng_solve(const double* T, int64_t B, const double* r, const double* p, const double* dinv, double* Ap, double* x,
+              CgScalars* sc, unsigned int* arrivals, unsigned int* status, cudaStream_t s, cudaError_t* e) {
+  *e = cudaSuccess;
+  const size_t smem = ng_solve_smem(B);
+  if (smem > kCgMaxSmem) return false;  // B > 9514
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  *e = cudaFuncSetAttribute(ng_cg_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (*e == cudaSuccess)
+    *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ng_cg_solve_kernel, kCgThreads, smem);
+  if (*e != cudaSuccess) return true;
+  int b = (int)B, rpc = (int)((B + sms - 1) / sms);  // rows per CTA, spread over every SM
+  if (per_sm < 1 || rpc > kCgThreads) return false;
+  const unsigned grid = ng_blocks(B, rpc);
+  *e = cudaMemsetAsync(arrivals, 0, sizeof(unsigned int), s);
+  if (*e != cudaSuccess) return true;
+  void* args[] = {&T, &b, &rpc, &r, &p, &dinv, &Ap, &x, &sc, &arrivals, &status};
+  *e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(ng_cg_solve_kernel), dim3(grid), dim3(kCgThreads),
+                                   args, smem, s);
+  return true;
+}
+
 }  // namespace
 
 // Workspace layout of natgrad_run (bytes), for B walkers and P parameters.
@@ -247,9 +429,11 @@ size_t natgrad_workspace(int64_t B, int64_t P) {
   o += 3 * ng_align((size_t)B * Pp * 4);        // Gc, TF32 high, TF32 low
   o += ng_align((size_t)kNgJobs * B * B * 4);  // Gram matrices of the chunks of one launch
   o += ng_align((size_t)B * B * 8);             // Gram matrix (FP64)
-  o += 6 * ng_align((size_t)B * 8);             // x, r, p, Ap, z, 1 / diag
+  o += 5 * ng_align((size_t)B * 8);             // x, r, p, z, 1 / diag
+  o += ng_align((size_t)2 * B * 8);             // Ap, two buffers
   o += 2 * ng_align((size_t)(mv_ctas + 1024) * 8);  // partials
   o += ng_align(sizeof(CgScalars));
+  o += ng_align(sizeof(unsigned int));          // arrivals at the solve's grid barrier
   return o;
 }
 
@@ -272,12 +456,13 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
   double* x = reinterpret_cast<double*>(take((size_t)B * 8));
   double* r = reinterpret_cast<double*>(take((size_t)B * 8));
   double* p = reinterpret_cast<double*>(take((size_t)B * 8));
-  double* Ap = reinterpret_cast<double*>(take((size_t)B * 8));
+  double* Ap = reinterpret_cast<double*>(take((size_t)2 * B * 8));
   double* z = reinterpret_cast<double*>(take((size_t)B * 8));
   double* dinv = reinterpret_cast<double*>(take((size_t)B * 8));
   double* partials = reinterpret_cast<double*>(take((size_t)(mv_ctas + 1024) * 8));
   double* partials2 = reinterpret_cast<double*>(take((size_t)(mv_ctas + 1024) * 8));
   CgScalars* sc = reinterpret_cast<CgScalars*>(take(sizeof(CgScalars)));
+  unsigned int* arrivals = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
 
   ng_colmean_kernel<<<ng_blocks(P, kNgThreads), kNgThreads, 0, s>>>(G, B, P, mean);
   ng_center_kernel<<<ng_blocks(B * Pp, kNgThreads), kNgThreads, 0, s>>>(G, mean, B, P, Pp, Gc);
@@ -300,12 +485,16 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
   }
   ng_symmetrize_kernel<<<ng_blocks(B * B, kNgThreads), kNgThreads, 0, s>>>(T, B);
   ng_cg_init_kernel<<<1, kNgThreads, 0, s>>>(w, B, T, x, r, p, dinv, sc, lam, tol, max_iter);
-  const unsigned up_ctas = ng_blocks(B, kNgThreads) < 1024 ? ng_blocks(B, kNgThreads) : 1024;
-  for (int it = 0; it < max_iter; ++it) {
-    ng_cg_matvec_kernel<<<(unsigned)mv_ctas, 32 * kNgRowWarps, 0, s>>>(T, B, p, Ap, sc, partials);
-    ng_cg_update_kernel<<<up_ctas, kNgThreads, 0, s>>>(B, x, r, z, dinv, p, Ap, sc, partials, partials2);
-    ng_cg_direction_kernel<<<up_ctas, kNgThreads, 0, s>>>(B, z, p, sc);
+  if (!ng_solve(T, B, r, p, dinv, Ap, x, sc, arrivals, status, s, &e)) {
+    // systems whose vectors do not fit one CTA's shared memory: three launches per iteration
+    const unsigned up_ctas = ng_blocks(B, kNgThreads) < 1024 ? ng_blocks(B, kNgThreads) : 1024;
+    for (int it = 0; it < max_iter; ++it) {
+      ng_cg_matvec_kernel<<<(unsigned)mv_ctas, 32 * kNgRowWarps, 0, s>>>(T, B, p, Ap, sc, partials);
+      ng_cg_update_kernel<<<up_ctas, kNgThreads, 0, s>>>(B, x, r, z, dinv, p, Ap, sc, partials, partials2);
+      ng_cg_direction_kernel<<<up_ctas, kNgThreads, 0, s>>>(B, z, p, sc);
+    }
   }
+  if (e != cudaSuccess) return e;
   ng_apply_kernel<<<ng_blocks(P, kNgThreads), kNgThreads, 0, s>>>(Gc, B, P, Pp, x, delta);
   if (stats) ng_stats_kernel<<<1, 1, 0, s>>>(sc, stats);
   return cudaGetLastError();

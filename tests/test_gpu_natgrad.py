@@ -157,3 +157,24 @@ def test_vmc_train_step_runs_and_is_reproducible():
         runs.append((th.clone(), r.clone()))
     assert not torch.equal(runs[0][0], th0)
     assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
+
+
+@pytest.mark.parametrize("B", [2, 9, 153, 300, 513])
+def test_one_kernel_solve_over_row_splits(B):
+    """The one-kernel conjugate gradients at row counts that leave remainders in its splits (rows
+    per CTA, groups of 8 and of 256 walkers), captured in a CUDA graph and replayed: the replay
+    gives the eager call's bits, and both the oracle's solution within the bound above."""
+    wl, h = _handle("lih_fp64")
+    G, w = _synthetic(B, h.P, 31 + B)
+    lam = _damping(G, 1e-1)
+    Gt = torch.tensor(G, dtype=torch.float32, device="cuda:0")
+    wt = torch.tensor(w, dtype=torch.float32, device="cuda:0")
+    eager, st = h.natural_gradient(Gt, wt, lam, max_iter=400, tol=1e-9)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        d, _ = h.natural_gradient(Gt, wt, lam, max_iter=400, tol=1e-9)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(d, eager) and float(st[1]) <= 1e-9
+    ref = oracle.natural_gradient(G, w, lam)
+    assert np.linalg.norm(d.cpu().numpy() - ref) <= 2e-3 * np.linalg.norm(ref)
