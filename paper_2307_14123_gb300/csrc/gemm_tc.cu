@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         int64_t rows, int n_out, int K, const float* __restrict__ bias, int bias_period,
                         float* __restrict__ Y, int64_t ldy, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(tc_smem_raw);
   uint8_t* sA = smem;
   uint8_t* sB = smem + TC_STAGES * TC_TILE_A;
   uint64_t* full = reinterpret_cast<uint64_t*>(sB + TC_STAGES * TC_TILE_B);
@@ -356,7 +356,7 @@ __device__ __forceinline__ void t3_epi_tile(const T3Jobs& jobs, int64_t tl, uint
 __global__ void __launch_bounds__(T3J_THREADS, 1)
     gemm_tf32x3_tc_kernel(const __grid_constant__ T3Jobs jobs, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(tc_smem_raw);
   // per stage: [x half 0, x half 1] (x_big after conversion), [x_small half 0, half 1], w_big, w_small
   uint8_t* sA = smem;
   uint8_t* sAs = sA + T3_STAGES * T3_SUB * T3_TILE_A;
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(T3_THREADS, 1)
                           int64_t rps, int64_t n_seg, int rb, int n_o, int n_a, int64_t splits, int64_t kps,
                           float* __restrict__ part, float* __restrict__ colpart, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(tc_smem_raw);
   uint8_t* sT = smem;                                   // [tstage][X tile, Y tile] as loaded: [32 rows][128]
   uint8_t* sO = sT + TN_TSTAGES * 2 * TN_TILE;          // [ostage][A hi, A lo, B hi, B lo] K-major, swizzled
   uint64_t* full = reinterpret_cast<uint64_t*>(sO + TN_OSTAGES * 4 * TN_TILE);

@@ -12,8 +12,15 @@ namespace dq {
 namespace tcp {
 
 constexpr long long kWaitCycles = 2000000000LL;   // ~1 s at 2 GHz
+// Longest sleep of one try_wait in ns: a waiting warp wakes when the phase completes, and polls
+// (issue slots that the working warps of its scheduler need) only this often.
+constexpr uint32_t kWaitHint = 1000000;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// The first 1024-byte boundary of a dynamic shared-memory block, by an offset: a pointer rounded
+// as an integer would lose its address space, and every access through it would be a generic one.
+__device__ __forceinline__ uint8_t* align1024(uint8_t* raw) { return raw + ((0u - smem_u32(raw)) & 1023u); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -27,9 +34,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   while (true) {
     uint32_t done;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kWaitHint)
         : "memory");
     if (done) return true;
     if (clock64() - t0 > kWaitCycles) return false;
