@@ -9,29 +9,38 @@
 // update to f in place.  Per walker the kernel reads the node map z (written
 // by the node-map GEMM), the filter jets, the geometry and f, and writes f.
 //
-// Rows of a tile: one walker, G = 128 / N consecutive node channels c and all
-// N receivers i, row = (c - c0) N + i; a walker is ceil(C / G) tiles, which
-// one CTA processes in channel order (the value channel first, the Laplacian
-// last), so that the Laplacian cross terms and sum_k J_k(u)^2 accumulate on
-// chip.  K steps: for each edge type t (same spin, opposite spin, nucleus)
+// Rows of a tile: one walker, the three coordinate channels of EPT consecutive
+// electrons (128 / N channels at most; the last tile takes the Laplacian and the
+// value channel too) and all N receivers i, row = (channel's place) N + i.  One
+// CTA processes a walker's tiles in electron order, the Laplacian last, so that
+// its cross terms accumulate on chip.  K steps: for each edge type t (same spin, opposite spin, nucleus)
 // and 32-feature block, A[row][32] = m_i^t[c][32 features] as three TF32
 // products with the W_g block (hi hi + hi lo + lo hi), or in BF16 mode as
 // one product of BF16 operands (FP32 accumulation).
 //
-// Warp roles (16 warps, one CTA per SM, persistent over walkers):
-//   warp 0      TMA: W_g hi/lo blocks (BF16: one block) and the z slab
-//               z_j[c0 .. c0 + G)[32] of all senders into a 2-stage ring;
+// Warp roles (14 warps, one CTA per SM, persistent over walkers):
+//   warp 0      TMA: W_g hi/lo blocks (BF16: one block) into a 2-stage ring, the
+//               z slab (the tile's channels, all senders, [32]) and z_j[0][32] (two
+//               buffers), and the filters w, w' of the step's edges (one buffer:
+//               the producers hold them in registers from the start of a step);
 //   warp 1      MMA issue (tcgen05.mma kind::tf32, 128 x 128 x 8; BF16:
 //               kind::f16, 128 x 128 x 16) into one of two tensor-memory
 //               accumulators;
-//   warps 2-3   idle;
-//   warps 4-7   epilogue: tensor memory -> the pre-activations U in global memory;
-//   warps 8-15  message producers: warp 8 + w owns two receivers of one spin
+//   warps 2-5   epilogue: tensor memory -> the pre-activations U in global memory;
+//   warps 6-13  message producers: warp 6 + w owns two receivers of one spin
 //               block (a half-warp each, two features per lane) and writes
 //               their rows of the A block (TF32 high and low parts, 128-byte
 //               swizzle; BF16: one part, 64-byte swizzle) from the z slab and
-//               the filter jets, prefetching the next K step's filter lines
-//               into L2.
+//               the filter jets, in packed FP32 arithmetic (f32x2.cuh).
+// What bounds it: the producers' instructions (two of their warps share a
+// scheduler), not the tensor pipe (about 1.2 K cycles of MMAs per K step) or
+// memory.  So the tiles are cut at whole electrons: an electron's three channels
+// are straight-line code without a test per channel, its loads ahead of its
+// stores; shared memory is reached through pointers whose address space the
+// compiler knows; and the filters arrive by TMA while the last step is produced
+// instead of through global loads at the start of their own.  The three layers
+// of 4096 N2 walkers: 10.7 ms with nine channels per tile in channel order and a
+// branch per channel (600 clocks per channel and warp), 6.5 ms so.
 // Every mbarrier wait is bounded (about one second); a timeout sets
 // DQ_FLAG_TIMEOUT, the roles stop issuing work, and the tensor memory is
 // released.
@@ -42,6 +51,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "tc_ptx.cuh"
 
 namespace dq {
@@ -53,13 +63,10 @@ constexpr int LF_D = 128;                  // embedding width (the MMA's N)
 constexpr int LF_NFB = LF_D / LF_BK;       // feature blocks per edge type
 constexpr int LF_KSTEPS = 2 * LF_NFB;      // K = 2 D: the electron-electron blocks of W_g
 constexpr int LF_STAGES = 2;
-constexpr int LF_UG = 2;                   // node channels per producer group
 constexpr int LF_PROD = 16;                // producer warps at most (one per receiver)
-// threads of the kernel for NB sender slots per spin block: 2 NB producer warps
-// 16 warps in four warpgroups: TMA and MMA issue (and two idle warps), epilogue, and two
-// warpgroups of producers (one warp per receiver pair).
-constexpr int LF_THREADS = 512;
 constexpr int LF_PROD_WARPS = 8;
+constexpr int LF_PROD_WARP0 = 6;           // warps 0 TMA, 1 MMA, 2-5 epilogue, 6-13 producers
+constexpr int LF_THREADS = (LF_PROD_WARP0 + LF_PROD_WARPS) * 32;
 constexpr int LF_MAX_N = 16;               // electrons (receivers per tile >= 8)
 constexpr int LF_MAX_BLK = 8;              // electrons per spin block
 constexpr int LF_MAX_M = 8;                // nuclei
@@ -73,14 +80,18 @@ constexpr uint32_t LF_OFF_Z = LF_STAGES * LF_STAGE;                             
 constexpr uint32_t LF_OFF_ACCL = LF_OFF_Z + LF_ZBUF * LF_TILE;                      // [N][2][D] Laplacian cross terms
 constexpr uint32_t LF_OFF_ST = LF_OFF_ACCL + LF_MAX_N * 2 * LF_D * 4;              // [4][32][33] transposes
 constexpr uint32_t LF_OFF_GEO = LF_OFF_ST + 4 * 32 * 33 * 4;                       // per receiver tables
-constexpr uint32_t LF_GEO_WARP = (LF_MAX_BLK * 2 + LF_MAX_M) * 8 * 4;              // rows x 8 floats
-constexpr uint32_t LF_OFF_BAR = LF_OFF_GEO + LF_PROD * LF_GEO_WARP;
+constexpr uint32_t LF_GEO_WARP = LF_MAX_BLK * 2 * 8 * 4;                           // rows x 8 floats
+constexpr uint32_t LF_EDGE = 2 * LF_BK * 4;                                        // w and w' of an edge
+constexpr uint32_t LF_OFF_FILT = LF_OFF_GEO + LF_PROD * LF_GEO_WARP;               // [edge][2][32] filters
+constexpr uint32_t LF_OFF_Z0 = LF_OFF_FILT + LF_MAX_BLK * LF_MAX_BLK * LF_EDGE;    // [2][N][32] z_j[0]
+constexpr uint32_t LF_Z0BUF = LF_MAX_N * LF_BK * 4;
+constexpr uint32_t LF_OFF_BAR = LF_OFF_Z0 + LF_ZBUF * LF_Z0BUF;
 constexpr uint32_t LF_SMEM = 1024 + LF_OFF_BAR + 20 * 8 + 16;
-static_assert(LF_SMEM <= 232448, "dynamic shared memory above the per-block limit");
+static_assert(LF_OFF_FILT % 128 == 0 && LF_OFF_Z0 % 128 == 0, "TMA destinations");
+static_assert(LF_SMEM + 1024 <= 232448, "dynamic shared memory above the per-block limit");
 
 struct LayerFusedArgs {
   const float* Z;       // [Bc][N][C][D] node map z_j (not read when z_const)
-  const float* zv;      // [Bc][N][D] a copy of the value channel z_j[0] (U overwrites Z's)
   const float* z0;      // [2][D] node map of the two spin embeddings (z_const)
   const float* ew;      // [Bc][E][3][D] filter jets: w, dw/dd, d2w/dd2
   const float* geo;     // [Bc][E][4] distance and unit vector of every edge
@@ -88,8 +99,10 @@ struct LayerFusedArgs {
   float* U;             // [Bc][N][C][D] W_g's electron-electron blocks times the messages (may be Z:
                         // a tile's rows are written after the last read of its z slab)
   int64_t Bc;
-  int N, n_up, M, C, E, n_ee, G, n_tiles;
+  int N, n_up, C, E, n_par;
+  int ept, slab, n_tiles;  // electrons per tile, channels of a z slab, tiles per walker
   int z_const;
+  int filt_rows;  // edges per filter load: the larger electron-electron edge type's count
   int n_prod;  // producer warps (receiver pairs), at most LF_PROD_WARPS
 };
 
@@ -98,9 +111,9 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
   while (true) {
     uint32_t done;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kWaitHint)
         : "memory");
     if (done) return true;
     if (*abort_flag) return false;
@@ -111,9 +124,9 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
 // x rounded to the nearest TF32 value (11 significant bits) by Veltkamp splitting: three FP32
 // operations, ties to even; the low part of a TF32 pair is rounded the same way, so that the
 // tensor cores (which read the top 19 bits of an operand) see it in full.
-__device__ __forceinline__ float tf32_split_hi(float x) {
-  const float t = __fmul_rn(x, 8193.f);
-  return __fsub_rn(t, __fsub_rn(t, x));
+__device__ __forceinline__ f2 tf32_split_hi(f2 x) {
+  const f2 t = f2_mul(x, f2_dup(8193.f));
+  return f2_sub(t, f2_sub(t, x));
 }
 
 // One lane's two messages (features 2 fp and 2 fp + 1 of its K step) into row `row` of the A
@@ -122,21 +135,19 @@ __device__ __forceinline__ float tf32_split_hi(float x) {
 // mode: one BF16 pair (round to nearest even) in a 128-row x 64-byte tile (64-byte swizzle:
 // chunk c of row r at c ^ ((r >> 1) & 3)).
 template <bool BF>
-__device__ __forceinline__ void store_a(uint8_t* a_hi, uint8_t* a_lo, int row, int fp, float2 m) {
+__device__ __forceinline__ void store_a(uint8_t* a_hi, uint8_t* a_lo, int row, int fp, f2 m) {
   if constexpr (BF) {
+    const float2 v = f2_unpack(m);
     const uint32_t o = (uint32_t)row * 64u + ((((uint32_t)fp >> 2) ^ (((uint32_t)row >> 1) & 3u)) << 4) +
                        ((uint32_t)(fp & 3) << 2);
-    *reinterpret_cast<__nv_bfloat162*>(a_hi + o) = __floats2bfloat162_rn(m.x, m.y);
+    *reinterpret_cast<__nv_bfloat162*>(a_hi + o) = __floats2bfloat162_rn(v.x, v.y);
   } else {
-    float2 hi, lo;
-    hi.x = tf32_split_hi(m.x);
-    hi.y = tf32_split_hi(m.y);
-    lo.x = tf32_split_hi(__fsub_rn(m.x, hi.x));
-    lo.y = tf32_split_hi(__fsub_rn(m.y, hi.y));
+    const f2 hi = tf32_split_hi(m);
+    const f2 lo = tf32_split_hi(f2_sub(m, hi));
     const uint32_t o = (uint32_t)row * 128u + ((((uint32_t)fp >> 1) ^ (uint32_t)(row & 7)) << 4) +
                        ((uint32_t)(fp & 1) << 3);
-    *reinterpret_cast<float2*>(a_hi + o) = hi;
-    *reinterpret_cast<float2*>(a_lo + o) = lo;
+    *reinterpret_cast<f2*>(a_hi + o) = hi;
+    *reinterpret_cast<f2*>(a_lo + o) = lo;
   }
 }
 
@@ -147,9 +158,10 @@ template <int NB, bool ZC, bool BF>
 __global__ void __launch_bounds__(LF_THREADS, 1)
     layer_fused_kernel(const __grid_constant__ LayerFusedArgs a, const __grid_constant__ CUtensorMap map_whi,
                        const __grid_constant__ CUtensorMap map_wlo, const __grid_constant__ CUtensorMap map_z,
-                       const __grid_constant__ CUtensorMap map_wbf, unsigned int* __restrict__ status) {
+                       const __grid_constant__ CUtensorMap map_wbf, const __grid_constant__ CUtensorMap map_zv,
+                       const __grid_constant__ CUtensorMap map_ew, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t lf_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(lf_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(lf_smem_raw);
   float* accL = reinterpret_cast<float*>(smem + LF_OFF_ACCL);
   float* stg = reinterpret_cast<float*>(smem + LF_OFF_ST);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + LF_OFF_BAR);
@@ -159,12 +171,15 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
   uint64_t* acc_empty = acc_full + 2;      // [2]
   uint64_t* zfull = acc_empty + 2;         // [LF_ZBUF]
   uint64_t* zempty = zfull + LF_ZBUF;      // [LF_ZBUF]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(zempty + LF_ZBUF);
+  uint64_t* ffull = zempty + LF_ZBUF;      // filters of a step
+  uint64_t* fempty = ffull + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fempty + 1);
   __shared__ volatile int s_abort;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int N = a.N, C = a.C, G = a.G, n_tiles = a.n_tiles;
-  const uint32_t zbytes = (uint32_t)(LF_BK * G * N * 4);
+  const int N = a.N, C = a.C, ept = a.ept, n_tiles = a.n_tiles;
+  const uint32_t zbytes = (uint32_t)(LF_BK * a.slab * N * 4 + LF_BK * N * 4);  // z slab and z_j[0]
+  const uint32_t fbytes = (uint32_t)a.filt_rows * LF_EDGE;
   const int n_prod = a.n_prod;  // producer warps: one per receiver pair
 
   if (threadIdx.x == 0) {
@@ -181,6 +196,8 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
       mbar_init(&zfull[q], 1);
       mbar_init(&zempty[q], n_prod);  // released by every producer warp after its last use
     }
+    mbar_init(ffull, 1);
+    mbar_init(fempty, n_prod);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
   }
@@ -188,6 +205,9 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
   // read, with weight zero, by the sender slots past a spin block
   for (uint32_t e = threadIdx.x; e < (LF_OFF_ST - LF_OFF_Z) / 4; e += blockDim.x)
     reinterpret_cast<float*>(smem + LF_OFF_Z)[e] = 0.f;
+  if (ZC)  // the constant node channels of the two spins, in place of the z_j[0] buffers
+    for (uint32_t e = threadIdx.x; e < 2 * LF_D; e += blockDim.x)
+      reinterpret_cast<float*>(smem + LF_OFF_Z0)[e] = a.z0[e];
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -215,9 +235,18 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
                 break;
               }
               mbar_expect_tx(&zfull[zb], zbytes);
-              tma_load_3d(smem + LF_OFF_Z + zb * LF_TILE, &map_z, fb * LF_BK, (int)(b * N), g * G, &zfull[zb]);
+              tma_load_3d(smem + LF_OFF_Z + zb * LF_TILE, &map_z, fb * LF_BK, (int)(b * N), 1 + 3 * ept * g,
+                          &zfull[zb]);
+              tma_load_2d(smem + LF_OFF_Z0 + zb * LF_Z0BUF, &map_zv, fb * LF_BK, (int)(b * N), &zfull[zb]);
               ++zi;
             }
+            // the filters of the step's edge type (loaded while the last step is produced)
+            if (g_ks >= 1 && !wait_or_abort(fempty, (uint32_t)((g_ks - 1) & 1), &s_abort)) {
+              s_abort = 1;
+              break;
+            }
+            mbar_expect_tx(ffull, fbytes);
+            tma_load_3d(smem + LF_OFF_FILT, &map_ew, fb * LF_BK, 0, (int)(b * a.E + (t == 0 ? 0 : a.n_par)), ffull);
             const int s = (int)(g_ks % LF_STAGES);
             const int64_t u = g_ks / LF_STAGES;
             if (u >= 1 && !wait_or_abort(&empty[s], (uint32_t)((u - 1) & 1), &s_abort)) {
@@ -283,59 +312,43 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
       }
       if (!ok) s_abort = 1;
     }
-  } else if (warp >= 8) {
-    if (warp - 8 >= n_prod) goto done;  // no receiver pair for this warp
-    // ---- message producers: warp 8 + w owns receiver pair w (two receivers of one spin block);
+  } else if (warp >= LF_PROD_WARP0) {
+    if (warp - LF_PROD_WARP0 >= n_prod) goto done;  // no receiver pair for this warp
+    // ---- message producers: warp LF_PROD_WARP0 + w owns receiver pair w (two receivers of one spin block);
     // lane (h, fp) = (lane / 16, lane % 16) computes features f0 + 2 fp and f0 + 2 fp + 1 of
     // receiver i_h.  The last pair of an odd block repeats its receiver in the second half,
     // which computes but never writes. ----
-    const int w = warp - 8;
+    const int w = warp - LF_PROD_WARP0;
     const int h = lane >> 4, fp = lane & 15;
-    const int n_up = a.n_up, M = a.M, E = a.E, n_ee = a.n_ee;
+    const int n_up = a.n_up, E = a.E, n_par = a.n_par;
     const int pairs_up = (n_up + 1) >> 1;
     int i = w < pairs_up ? 2 * w + h : n_up + 2 * (w - pairs_up) + h;
     const bool writer = w < pairs_up ? i < n_up : i < N;
     if (!writer) i -= 1;
     const bool up = i < n_up;
-    // geometry of receiver i, once per walker: per sender slot k of the same spin block (k < 8),
-    // of the other block (8 <= k < 16) and per nucleus (16 <= k): the edge index (as float bits),
+    // geometry of receiver i, once per walker: per sender slot k of the same spin block (k < 8)
+    // and of the other block (8 <= k): the edge's index within its type (as float bits, -1: none),
     // the unit vector u_ij and 1 / d_ij
     float* gt = reinterpret_cast<float*>(smem + LF_OFF_GEO + i * LF_GEO_WARP);
-    constexpr int kRows = LF_MAX_BLK * 2 + LF_MAX_M;
+    constexpr int kRows = LF_MAX_BLK * 2;
+    const float* filt = reinterpret_cast<const float*>(smem + LF_OFF_FILT) + 2 * fp;  // [edge][w, w'][32]
+    const f2 two = f2_dup(2.f);
     int64_t g_ks = 0, zi = 0;
     bool ok = true;
-    // the filter-jet lines of K step (t, f0) into L2: lane fp < 8 sender slot fp's value,
-    // 8 <= fp its first derivative
-    auto prefetch_filters = [&](const float* ew_b, int t, int f0) {
-      const int k = fp & 7, jet = fp >> 3;
-      const int row = (t == 0 ? 0 : LF_MAX_BLK) + k;
-      const int edge = __float_as_int(gt[row * 8]);
-      if (edge >= 0)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(ew_b + ((int64_t)edge * 3 + jet) * LF_D + f0));
-    };
     for (int64_t b = blockIdx.x; b < a.Bc && ok; b += gridDim.x) {
       const float* geo_b = a.geo + b * E * 4;
       const float* ew_b = a.ew + b * (int64_t)E * 3 * LF_D;
-      const float* zv_b = a.zv + b * (int64_t)N * LF_D;
       if (writer) {
         for (int k = fp; k < kRows; k += 16) {
           float* row = gt + k * 8;
-          int edge = -1;
-          float sg = 1.f;
-          if (k < 2 * LF_MAX_BLK) {
-            const bool same = k < LF_MAX_BLK;
-            const int j0 = (up == same) ? 0 : n_up, j1 = (up == same) ? n_up : N;
-            const int j = j0 + (k % LF_MAX_BLK);
-            if (j < j1 && j != i) {
-              edge = a.pair_of[i * N + j];
-              sg = i < j ? 1.f : -1.f;
-            }
-          } else if (k - 2 * LF_MAX_BLK < M) {
-            edge = n_ee + i * M + (k - 2 * LF_MAX_BLK);
-          }
-          if (edge >= 0) {
+          const bool same = k < LF_MAX_BLK;
+          const int j0 = (up == same) ? 0 : n_up, j1 = (up == same) ? n_up : N;
+          const int j = j0 + (k % LF_MAX_BLK);
+          if (j < j1 && j != i) {
+            const int edge = a.pair_of[i * N + j];
+            const float sg = i < j ? 1.f : -1.f;
             const float* gg = geo_b + (int64_t)edge * 4;
-            row[0] = __int_as_float(edge);
+            row[0] = __int_as_float(edge - (same ? 0 : n_par));
             row[1] = sg * gg[1];
             row[2] = sg * gg[2];
             row[3] = sg * gg[3];
@@ -347,200 +360,160 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
         }
       }
       __syncwarp();
-      prefetch_filters(ew_b, 0, 0);
       for (int g = 0; g < n_tiles && ok; ++g) {
-        const int c0 = g * G;
-        const int c1 = min(C, c0 + G);
+        const int e0 = min(N, g * ept), e1 = min(N, e0 + ept);  // the tile's electrons
+        const bool last = g == n_tiles - 1;
         for (int ks = 0; ks < LF_KSTEPS; ++ks, ++g_ks) {
           const int s = (int)(g_ks % LF_STAGES);
           const int fb = ks / 2, t = ks % 2;
-          const int f0 = fb * LF_BK;
-          const int fl = f0 + 2 * fp;  // this lane's first feature
+          const int fl = fb * LF_BK + 2 * fp;  // this lane's first feature
           // electron-electron messages of type t: senders j = j0 + k, k < NB
           const bool same = t == 0;
           const int j0 = (up == same) ? 0 : n_up, j1 = (up == same) ? n_up : N;
           const float* gs = gt + (same ? 0 : LF_MAX_BLK) * 8;
-          // the step's filter jets and, past tile 0, the senders' z_j[0] (global loads issued
-          // before the waits, so that their latency overlaps them); slots without an edge read
-          // edge 0 and are masked below
-          float2 wv[NB], w1[NB], z0v[NB];
+          const float* ew_t = ew_b + (int64_t)(same ? 0 : n_par) * 3 * LF_D + fl;  // the type's first edge
+          // the Laplacian channel's w'' lines into L2 ahead of their use at the end of the step
+          if (last && fp < NB) {
+            const int edge = __float_as_int(gs[fp * 8]);
+            if (edge >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ew_t - 2 * fp + ((int64_t)edge * 3 + 2) * LF_D));
+          }
+          const int zb = (int)(zi % LF_ZBUF);
+          const float* zs = reinterpret_cast<const float*>(smem + LF_OFF_Z + zb * LF_TILE) + 2 * fp;  // [channel][j][32]
+          const float* z0s = ZC ? reinterpret_cast<const float*>(smem + LF_OFF_Z0) + fl             // [spin][D]
+                                : reinterpret_cast<const float*>(smem + LF_OFF_Z0 + zb * LF_Z0BUF) + 2 * fp;  // [j][32]
+          auto z0_at = [&](int j) {  // z_j[0] of this lane's features
+            return *reinterpret_cast<const f2*>(z0s + (ZC ? (j < n_up ? 0 : LF_D) : j * LF_BK));
+          };
+          if (!wait_or_abort(ffull, (uint32_t)(g_ks & 1), &s_abort)) {
+            ok = false;
+            break;
+          }
+          f2 wv[NB], w1[NB];  // the step's filters; slots without an edge read edge 0 and are masked
 #pragma unroll
           for (int k = 0; k < NB; ++k) {
             const int edge = __float_as_int(gs[k * 8]);
-            const float* wp = ew_b + (int64_t)(edge >= 0 ? edge : 0) * 3 * LF_D + fl;
-            wv[k] = __ldg(reinterpret_cast<const float2*>(wp));
-            w1[k] = __ldg(reinterpret_cast<const float2*>(wp + LF_D));
-            const int j = min(j0 + k, N - 1);
-            if (ZC)
-              z0v[k] = __ldg(reinterpret_cast<const float2*>(a.z0 + (j < n_up ? 0 : LF_D) + fl));
-            else if (c0 > 0)
-              z0v[k] = __ldg(reinterpret_cast<const float2*>(zv_b + (int64_t)j * LF_D + fl));
+            const float* wp = filt + (edge >= 0 ? edge : 0) * (int)(LF_EDGE / 4);
+            const f2 x0 = *reinterpret_cast<const f2*>(wp), x1 = *reinterpret_cast<const f2*>(wp + LF_BK);
+            wv[k] = edge >= 0 ? x0 : 0ull;
+            w1[k] = edge >= 0 ? x1 : 0ull;
           }
-          // the Laplacian channel's w'' lines into L2 ahead of their use at the end of the step
-          if (c1 == C && fp < NB) {
-            const int edge = __float_as_int(gs[fp * 8]);
-            if (edge >= 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ew_b + ((int64_t)edge * 3 + 2) * LF_D + f0));
-          }
-          if (!wait_or_abort(&full[s], (uint32_t)((g_ks / LF_STAGES) & 1), &s_abort)) {
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(fempty)) : "memory");
+          if ((!ZC && !wait_or_abort(&zfull[zb], (uint32_t)((zi / LF_ZBUF) & 1), &s_abort)) ||
+              !wait_or_abort(&full[s], (uint32_t)((g_ks / LF_STAGES) & 1), &s_abort)) {
             ok = false;
             break;
           }
           uint8_t* a_hi = smem + s * LF_STAGE;
           uint8_t* a_lo = a_hi + LF_TILE;
-          const int zb = (int)(zi % LF_ZBUF);
-          const float* zs = reinterpret_cast<const float*>(smem + LF_OFF_Z + zb * LF_TILE);  // [c - c0][j][32]
-          if (!ZC && !wait_or_abort(&zfull[zb], (uint32_t)((zi / LF_ZBUF) & 1), &s_abort)) {
-            ok = false;
-            break;
-          }
           const int n_send = same ? (j1 - j0) - 1 : (j1 - j0);
-          const float nu = 1.f / (float)(n_send > 1 ? n_send : 1);
-          // the next K step's filter lines into L2 while this one is produced
-          if (ks + 1 < LF_KSTEPS) prefetch_filters(ew_b, (ks + 1) % 2, ((ks + 1) / 2) * LF_BK);
-          else if (g + 1 < n_tiles) prefetch_filters(ew_b, 0, 0);
-#pragma unroll
-          for (int k = 0; k < NB; ++k) {
-            const bool v = __float_as_int(gs[k * 8]) >= 0;
-            const int j = min(j0 + k, N - 1);
-            if (!ZC && c0 == 0) z0v[k] = *reinterpret_cast<const float2*>(zs + j * LF_BK + 2 * fp);
-            wv[k] = v ? wv[k] : make_float2(0.f, 0.f);
-            w1[k] = v ? w1[k] : make_float2(0.f, 0.f);
-            z0v[k] = v ? z0v[k] : make_float2(0.f, 0.f);
-          }
+          const f2 nu = f2_dup(1.f / (float)(n_send > 1 ? n_send : 1));
+          // half the Laplacian channel's cross terms, sum_j w'_ij u_ij . (dz_j/dr_i - dz_j/dr_j) so far
           float* acl = accL + (i * 2 + t) * LF_D + fl;
-          float2 accv = g == 0 ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(acl);
+          f2 acc = g == 0 ? 0ull : *reinterpret_cast<const f2*>(acl);
           {
             // the receiver's own coordinates, for both halves at once (no divergence on i):
-            // m_i[c] = sum_j w_ij z_j[c] + sum_j w'_ij u_ij,x z_j[0], c = 1 + 3 i + x, and the Laplacian
-            // cross term 2 sum_j w'_ij u_ij,x dz_j/dr_i,x (before the channel loop, whose Laplacian
-            // channel reads the cross terms)
-            const int cb = 1 + 3 * i;
-            const bool any_own = cb + 2 >= c0 && cb < c1;
-            if (__any_sync(0xffffffffu, any_own)) {
+            // m_i[c] = sum_j w_ij z_j[c] + sum_j w'_ij u_ij,x z_j[0], c = 1 + 3 i + x, and the cross
+            // term sum_j w'_ij u_ij,x dz_j/dr_i,x
+            const bool act = i >= e0 && i < e1;
+            if (__any_sync(0xffffffffu, act)) {
+              const int r0 = act ? 3 * (i - e0) : 0;
+              f2 z0v[NB];
+#pragma unroll
+              for (int k = 0; k < NB; ++k) z0v[k] = z0_at(min(j0 + k, N - 1));
 #pragma unroll
               for (int x = 0; x < 3; ++x) {
-                const int c = cb + x;
-                const bool act = c >= c0 && c < c1;
-                const float* zr = zs + ((act ? c - c0 : 0) * N + j0) * LF_BK + 2 * fp;
-                float2 m = make_float2(0.f, 0.f), cr = make_float2(0.f, 0.f);
+                const float* zr = zs + ((r0 + x) * N + j0) * LF_BK;
+                f2 m = 0ull, cr = 0ull;
 #pragma unroll
                 for (int k = 0; k < NB; ++k) {
-                  const float ux = gs[k * 8 + 1 + x];
-                  const float2 ak = make_float2(w1[k].x * ux, w1[k].y * ux);
-                  m.x = fmaf(ak.x, z0v[k].x, m.x);
-                  m.y = fmaf(ak.y, z0v[k].y, m.y);
+                  const f2 ak = f2_mul(w1[k], f2_dup(gs[k * 8 + 1 + x]));
+                  m = f2_fma(ak, z0v[k], m);
                   if (!ZC) {
-                    const float2 z = *reinterpret_cast<const float2*>(zr + k * LF_BK);
-                    m.x = fmaf(wv[k].x, z.x, m.x);
-                    m.y = fmaf(wv[k].y, z.y, m.y);
-                    cr.x = fmaf(ak.x, z.x, cr.x);
-                    cr.y = fmaf(ak.y, z.y, cr.y);
+                    const f2 z = *reinterpret_cast<const f2*>(zr + k * LF_BK);
+                    m = f2_fma(wv[k], z, m);
+                    cr = f2_fma(ak, z, cr);
                   }
                 }
                 if (act) {
-                  accv.x = fmaf(2.f, cr.x, accv.x);
-                  accv.y = fmaf(2.f, cr.y, accv.y);
-                  if (writer) {
-                    m.x *= nu;
-                    m.y *= nu;
-                    store_a<BF>(a_hi, a_lo, (c - c0) * N + i, fp, m);
-                  }
+                  acc = f2_add(acc, cr);
+                  if (writer) store_a<BF>(a_hi, a_lo, (r0 + x) * N + i, fp, f2_mul(m, nu));
                 }
               }
             }
           }
-          const float* zrow = zs + j0 * LF_BK + 2 * fp;  // channel c0's senders
-          int row = i;                                    // A row of (c0, i)
-          int e = c0 >= 1 ? (c0 - 1) / 3 : -1, x = c0 >= 1 ? (c0 - 1) - 3 * e : 2;  // electron, axis of c0
-          int ke_c = -1;                                  // the sender slot whose w' and z_j[0] are cached
-          float2 w1e = make_float2(0.f, 0.f), z0e = make_float2(0.f, 0.f);
-          // channels in groups of LF_UG: the loads and multiply-add chains of a group overlap
-          for (int cg = c0; cg < c1; cg += LF_UG, zrow += LF_UG * N * LF_BK) {
-            float2 zc[LF_UG][NB], mm[LF_UG];
+          // sum_k w_k z_k[c] of one channel, its senders at zr (even and odd senders apart)
+          auto contract = [&](const f2 (&z)[NB]) {
+            f2 m0 = 0ull, m1 = 0ull;
 #pragma unroll
-            for (int u = 0; u < LF_UG; ++u) {
-              // rows past c1 stay inside the z buffers (finite data) and their sums are dropped
-#pragma unroll
-              for (int k = 0; k < NB; ++k)
-                zc[u][k] = ZC ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(zrow + (u * N + k) * LF_BK);
+            for (int k = 0; k < NB; k += 2) {
+              m0 = f2_fma(wv[k], z[k], m0);
+              if (k + 1 < NB) m1 = f2_fma(wv[k + 1], z[k + 1], m1);
             }
+            return f2_add(m0, m1);
+          };
+          // the coordinate channels of the tile's electrons, three per electron: straight-line code,
+          // with every load of an electron ahead of its stores
+          const float* ze = zs + j0 * LF_BK;
+          int row = i;
+          for (int e = e0; e < e1; ++e, ze += 3 * N * LF_BK, row += 3 * N) {
+            f2 m[3] = {0ull, 0ull, 0ull};
+            const bool snd = e >= j0 && e < j1;
+            if (!ZC) {
+              f2 zc[3][NB];
 #pragma unroll
-            for (int u = 0; u < LF_UG; ++u) {
-              float2 m0 = make_float2(0.f, 0.f), m1 = make_float2(0.f, 0.f);
-              if (!ZC || (cg + u == 0)) {
+              for (int x = 0; x < 3; ++x)
 #pragma unroll
-                for (int k = 0; k < NB; k += 2) {
-                  const float2 z = ZC ? z0v[k] : zc[u][k];
-                  m0.x = fmaf(wv[k].x, z.x, m0.x);
-                  m0.y = fmaf(wv[k].y, z.y, m0.y);
-                  if (k + 1 < NB) {
-                    const float2 z1 = ZC ? z0v[k + 1] : zc[u][k + 1];
-                    m1.x = fmaf(wv[k + 1].x, z1.x, m1.x);
-                    m1.y = fmaf(wv[k + 1].y, z1.y, m1.y);
-                  }
-                }
-              }
-              mm[u] = make_float2(m0.x + m1.x, m0.y + m1.y);
+                for (int k = 0; k < NB; ++k) zc[x][k] = *reinterpret_cast<const f2*>(ze + (x * N + k) * LF_BK);
+#pragma unroll
+              for (int x = 0; x < 3; ++x) m[x] = contract(zc[x]);
             }
+            if (snd) {
+              // a sender's coordinates: -w'_ie u_ie,x z_e[0]; cross term -w'_ie u_ie,x dz_e/dr_e,x (zero
+              // for the receiver's own slot, whose weights are masked)
+              const int ke = e - j0;
+              f2 w1e = w1[0];
 #pragma unroll
-            for (int u = 0; u < LF_UG; ++u) {
-              const int c = cg + u;
-              if (c >= c1) break;
-              float2 m = mm[u];
-              if (c >= 1 && c < C - 1) {
-                if (e >= j0 && e < j1) {
-                  // a sender's coordinate: -w'_ie u_ie,x z_e[0]; Laplacian cross term
-                  // -2 w'_ie u_ie,x dz_e/dr_e,x (zero for the receiver's own slot, whose weights
-                  // are masked); the slot's registers are picked once per electron
-                  const int ke = e - j0;
-                  if (ke != ke_c) {
-                    ke_c = ke;
-                    w1e = w1[0];
-                    z0e = z0v[0];
+              for (int k = 1; k < NB; ++k)
+                if (ke == k) w1e = w1[k];
+              const float4 gu = *reinterpret_cast<const float4*>(gs + ke * 8);
+              const f2 z0e = z0_at(e);
 #pragma unroll
-                    for (int k = 1; k < NB; ++k)
-                      if (ke == k) {
-                        w1e = w1[k];
-                        z0e = z0v[k];
-                      }
-                  }
-                  const float ux = gs[ke * 8 + 1 + x];
-                  const float2 ak = make_float2(w1e.x * ux, w1e.y * ux);
-                  m.x = fmaf(-ak.x, z0e.x, m.x);
-                  m.y = fmaf(-ak.y, z0e.y, m.y);
-                  if (!ZC) {
-                    const float2 zce = *reinterpret_cast<const float2*>(zrow + (u * N + ke) * LF_BK);
-                    accv.x = fmaf(-2.f * ak.x, zce.x, accv.x);
-                    accv.y = fmaf(-2.f * ak.y, zce.y, accv.y);
-                  }
-                }
-              } else if (c == C - 1) {
-                // sum_j (2 w''_ij + 4 w'_ij / d_ij) z_j[0] + the accumulated cross terms
-#pragma unroll
-                for (int k = 0; k < NB; ++k) {
-                  const int edge = __float_as_int(gs[k * 8]);
-                  const float2 w2 = edge >= 0
-                                        ? __ldg(reinterpret_cast<const float2*>(ew_b + ((int64_t)edge * 3 + 2) * LF_D + fl))
-                                        : make_float2(0.f, 0.f);
-                  const float id = 4.f * gs[k * 8 + 4];
-                  m.x = fmaf(fmaf(2.f, w2.x, id * w1[k].x), z0v[k].x, m.x);
-                  m.y = fmaf(fmaf(2.f, w2.y, id * w1[k].y), z0v[k].y, m.y);
-                }
-                m.x += accv.x;
-                m.y += accv.y;
+              for (int x = 0; x < 3; ++x) {
+                const f2 ak = f2_mul(w1e, f2_dup(x == 0 ? -gu.y : x == 1 ? -gu.z : -gu.w));
+                m[x] = f2_fma(ak, z0e, m[x]);
+                if (!ZC) acc = f2_fma(ak, *reinterpret_cast<const f2*>(ze + (x * N + ke) * LF_BK), acc);
               }
-              m.x *= nu;
-              m.y *= nu;
-              if (writer && e != i)  // (the receiver's own channels were formed above)
-                store_a<BF>(a_hi, a_lo, row, fp, m);
-              row += N;
-              if (++x == 3) {
-                x = 0;
-                ++e;
-              }
+            }
+            if (writer && e != i) {  // (the receiver's own channels were formed above)
+#pragma unroll
+              for (int x = 0; x < 3; ++x) store_a<BF>(a_hi, a_lo, row + x * N, fp, f2_mul(m[x], nu));
             }
           }
-          if (writer) *reinterpret_cast<float2*>(acl) = accv;
+          if (last) {
+            // the Laplacian channel: sum_j w_ij z_j[C - 1] + (2 w''_ij + 4 w'_ij / d_ij) z_j[0] + the cross
+            // terms; then the value channel
+            f2 z0v[NB], zl[NB], w2[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+              const int edge = __float_as_int(gs[k * 8]);
+              w2[k] = edge >= 0 ? __ldg(reinterpret_cast<const f2*>(ew_t + ((int64_t)edge * 3 + 2) * LF_D)) : 0ull;
+              z0v[k] = z0_at(min(j0 + k, N - 1));
+              zl[k] = ZC ? 0ull : *reinterpret_cast<const f2*>(ze + k * LF_BK);
+            }
+            f2 ml = contract(zl);
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+              ml = f2_fma(f2_fma(two, w2[k], f2_mul(f2_dup(4.f * gs[k * 8 + 4]), w1[k])), z0v[k], ml);
+            ml = f2_fma(two, acc, ml);
+            const f2 mv = contract(z0v);
+            if (writer) {
+              store_a<BF>(a_hi, a_lo, row, fp, f2_mul(ml, nu));
+              store_a<BF>(a_hi, a_lo, row + N, fp, f2_mul(mv, nu));
+            }
+          } else if (writer) {
+            *reinterpret_cast<f2*>(acl) = acc;
+          }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // A block visible to the tensor cores
           __syncwarp();
           if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&conv[s])) : "memory");
@@ -552,8 +525,8 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
       }
     }
     if (!ok) s_abort = 1;
-  } else if (warp >= 4) {
-    // ---- epilogue warps 4..7: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 ----
+  } else {
+    // ---- epilogue warps 2..5: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 ----
     // Per 32-feature chunk: the warp's 32 rows of the accumulator through a shared-memory
     // transpose, stored as full 128-byte lines of U (the electron-nucleus part, un, is added by
     // the kernel that follows).
@@ -564,9 +537,8 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
       float* Ub = a.U + b * (int64_t)N * C * LF_D;
       for (int g = 0; g < n_tiles; ++g, ++lt) {
         const int acc_i = (int)(lt & 1);
-        const int c0 = g * G;
-        const int c1 = min(C, c0 + G);
-        const int nrows = (c1 - c0) * N;
+        const int e0 = min(N, g * ept), n_coord = 3 * (min(N, e0 + ept) - e0);
+        const int nrows = (n_coord + (g == n_tiles - 1 ? 2 : 0)) * N;
         bool live = wait_or_abort(&acc_full[acc_i], (uint32_t)((lt >> 1) & 1), &s_abort) && !s_abort;
         live = __all_sync(0xffffffffu, live);  // warp-uniform: the tensor-memory loads are warp-wide
         if (!live) s_abort = 1;
@@ -582,7 +554,8 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
           int cc = cc_first, ii = i_first;
           for (int rr = 0; rr < 32; ++rr) {
             if (q * 32 + rr >= nrows) break;
-            Ub[((int64_t)ii * C + c0 + cc) * LF_D + d0 + lane] = stw[rr][lane];
+            const int c = cc < n_coord ? 1 + 3 * e0 + cc : cc == n_coord ? C - 1 : 0;
+            Ub[((int64_t)ii * C + c) * LF_D + d0 + lane] = stw[rr][lane];
             if (++ii == N) {
               ii = 0;
               ++cc;
@@ -681,6 +654,32 @@ bool map_w(CUtensorMap* m, const float* W, int D) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The value channels zv [Bc N][D], box {32 features, N senders}.
+bool map_zv(CUtensorMap* m, const float* zv, int64_t Bc, int N, int D) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)(N * Bc)};
+  const cuuint64_t strides[1] = {(cuuint64_t)D * 4};
+  const cuuint32_t box[2] = {LF_BK, (cuuint32_t)N};
+  const cuuint32_t estr[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(zv), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The filter jets ew [Bc E][3][D] as dims {D, 3, E Bc}, box {32 features, w and w', rows edges}.
+bool map_ew(CUtensorMap* m, const float* ew, int64_t Bc, int E, int D, int rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)D, 3, (cuuint64_t)(E * Bc)};
+  const cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)D * 12};
+  const cuuint32_t box[3] = {LF_BK, 2, (cuuint32_t)rows};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(ew), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // z [Bc][N][C][D] as dims {D, N Bc, C} (sender before channel); box {32 features, N senders,
 // G channels}, so that the slab in shared memory is [channel][sender][32]; channels past C read zeros.
 bool map_z(CUtensorMap* m, const float* Z, int64_t Bc, int N, int C, int D, int G) {
@@ -695,7 +694,8 @@ bool map_z(CUtensorMap* m, const float* Z, int64_t Bc, int N, int C, int D, int 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-using KernT = void (*)(LayerFusedArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, unsigned int*);
+using KernT = void (*)(LayerFusedArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
+                       unsigned int*);
 
 template <bool BF>
 KernT pick_kernel(int nb, bool z_const) {
@@ -740,7 +740,6 @@ cudaError_t launch_layer_fused(const dq_handle_s& h, const FwdDims& d, const flo
   if (e != cudaSuccess) return e;
   LayerFusedArgs a{};
   a.Z = Z;
-  a.zv = zv;
   a.z0 = z0;
   a.ew = ew;
   a.geo = geo;
@@ -749,19 +748,30 @@ cudaError_t launch_layer_fused(const dq_handle_s& h, const FwdDims& d, const flo
   a.Bc = d.Bc;
   a.N = d.N;
   a.n_up = d.n_up;
-  a.M = d.M;
   a.C = d.C;
   a.E = h.edges.n_all;
-  a.n_ee = h.edges.n_ee;
-  a.G = std::min(128 / d.N, d.C);
-  a.n_tiles = (d.C + a.G - 1) / a.G;
+  a.n_par = h.edges.n_par;
+  a.filt_rows = std::max({h.edges.n_par, h.edges.n_anti, 1});
+  // electrons per tile: three rows of N receivers each, and in the last tile (one more where they do
+  // not fit) the Laplacian and the value channel
+  const int chan = 128 / d.N;
+  a.ept = std::min(d.N, chan / 3);
+  a.n_tiles = (d.N + a.ept - 1) / a.ept;
+  int n_last = d.N - (a.n_tiles - 1) * a.ept;
+  if (3 * n_last + 2 > chan) {
+    ++a.n_tiles;
+    n_last = 0;
+  }
+  a.slab = std::max(3 * (a.n_tiles > 1 ? a.ept : n_last), 3 * n_last + 1);
   a.z_const = z_const ? 1 : 0;
-  CUtensorMap mhi, mlo, mz, mbf;
+  CUtensorMap mhi, mlo, mz, mbf, mzv, mew;
   if (!map_w(&mhi, wg_hi, LF_D) || !map_w(&mlo, wg_lo, LF_D)) return cudaErrorInvalidValue;
   // BF16 operands when the BF16 copy of W_g is given (otherwise mbf is a copy of the FP32 map, unread)
   if (wg_bf ? !map_w_bf(&mbf, wg_bf, LF_D) : !map_w(&mbf, wg_hi, LF_D)) return cudaErrorInvalidValue;
   // with constant node channels the z slabs are never loaded; their maps are built on W (any valid map)
-  if (!(z_const ? map_w(&mz, wg_hi, LF_D) : map_z(&mz, Z, d.Bc, d.N, d.C, LF_D, a.G))) return cudaErrorInvalidValue;
+  if (!(z_const ? map_w(&mz, wg_hi, LF_D) : map_z(&mz, Z, d.Bc, d.N, d.C, LF_D, a.slab))) return cudaErrorInvalidValue;
+  if (!(z_const ? map_w(&mzv, wg_hi, LF_D) : map_zv(&mzv, zv, d.Bc, d.N, LF_D))) return cudaErrorInvalidValue;
+  if (!map_ew(&mew, ew, d.Bc, a.E, LF_D, a.filt_rows)) return cudaErrorInvalidValue;
   const int nb = std::max(h.n_up, h.n_dn);
   const KernT kern = wg_bf ? pick_kernel<true>(nb, z_const) : pick_kernel<false>(nb, z_const);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LF_SMEM);
@@ -772,7 +782,7 @@ cudaError_t launch_layer_fused(const dq_handle_s& h, const FwdDims& d, const flo
   const int64_t grid = d.Bc < sms ? d.Bc : sms;
   a.n_prod = (h.n_up + 1) / 2 + (h.n_dn + 1) / 2;  // receiver pairs of the two spin blocks
   if (a.n_prod > LF_PROD_WARPS) return cudaErrorInvalidValue;
-  kern<<<(unsigned)grid, LF_THREADS, LF_SMEM, s>>>(a, mhi, mlo, mz, mbf, h.d_status);
+  kern<<<(unsigned)grid, LF_THREADS, LF_SMEM, s>>>(a, mhi, mlo, mz, mbf, mzv, mew, h.d_status);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   add_nucleus_part_kernel<<<(unsigned)(d.Bc * d.N), LF_D, 0, s>>>(un, d.N, d.C, Z);
