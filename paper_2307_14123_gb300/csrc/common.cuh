@@ -258,7 +258,14 @@ struct T3JobDesc {
   int64_t ldy, y_seg_stride;
   bool accumulate;
   int64_t ldw = 0;  // row pitch of Wbig / Wsmall in elements (0: K)
+  // W itself (unsplit) in Wbig, split in shared memory like X (Wsmall unused); for products whose W
+  // is used once, so that a split copy of it in memory would cost more than splitting its tiles.
+  // All jobs of a call alike.
+  bool raw_w = false;
+  bool tri = false;  // Y square: only the tiles that reach row >= column (the rest of Y is not written)
 };
+// Output tiles of such a job: all, or (tri) those that reach row >= column.
+int64_t gemm_tf32x3_tiles(int64_t rows, int64_t cols, bool tri);
 cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* jobs, int n, unsigned int* status, cudaStream_t s);
 // TF32 high / low parts of the transpose of W [rows][cols] (for products X W).
 cudaError_t split_tf32_t(const float* W, int rows, int cols, float* big, float* small, cudaStream_t s);

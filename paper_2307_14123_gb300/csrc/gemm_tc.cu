@@ -26,6 +26,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -276,7 +278,7 @@ struct T3Fields {
   float* Y;
   int64_t seg_rows, n_seg, ldy, y_seg_stride;
   int64_t rb_per_seg, n_mblk, tile_end;  // tile_end: tiles of jobs 0 .. this one
-  int rb, sb, n_out, nk, n_tiles_n, bias_period, accumulate;
+  int rb, sb, n_out, nk, n_tiles_n, bias_period, accumulate, tri;
 };
 struct T3Job {
   CUtensorMap a, bb, bs;  // X (segmented rows), W big, W small
@@ -293,15 +295,46 @@ __device__ __forceinline__ int t3_job(const T3Fields* sj, int n, int64_t t, int6
   tl = t - (m > 0 ? sj[m - 1].tile_end : 0);
   return m;
 }
-// TMA loads of one K block of job M's tile (A blocks of T3_SUB segments, W big and small).
-template <int M>
+// Row-block pair mp and column block nt of a job's tile tl.  A triangular job lists, for every row
+// pair (256 rows), the 2 mp + 2 column blocks up to its last row, mp (mp + 1) tiles before it.
+__device__ __forceinline__ void t3_tile(int64_t tl, int n_tiles_n, int tri, int64_t& mp, int& nt) {
+  static_assert(T3_SUB * TC_BM == 2 * TC_BN, "the triangle's tile count per row pair");
+  if (tri) {
+    int m = (int)((sqrtf(4.f * (float)tl + 1.f) - 1.f) * 0.5f);
+    while ((int64_t)m * (m + 1) > tl) --m;
+    while ((int64_t)(m + 1) * (m + 2) <= tl) ++m;
+    mp = m;
+    nt = (int)(tl - (int64_t)m * (m + 1));
+  } else {
+    mp = tl / n_tiles_n;
+    nt = (int)(tl % n_tiles_n);
+  }
+}
+// x split into TF32 parts, four values at a time.
+__device__ __forceinline__ void t3_split4(float4* src, float4* dst) {
+  const float4 x = *src;
+  float4 b, sm;
+  b.x = tf32_rn(x.x);
+  b.y = tf32_rn(x.y);
+  b.z = tf32_rn(x.z);
+  b.w = tf32_rn(x.w);
+  sm.x = tf32_rn(x.x - b.x);
+  sm.y = tf32_rn(x.y - b.y);
+  sm.z = tf32_rn(x.z - b.z);
+  sm.w = tf32_rn(x.w - b.w);
+  *src = b;
+  *dst = sm;
+}
+// TMA loads of one K block of job M's tile (A blocks of T3_SUB segments, W big and small, or
+// (RAW) W itself into the big part's buffer).
+template <int M, bool RAW>
 __device__ __forceinline__ void t3_issue(const T3Jobs& jobs, uint8_t* a_dst, uint8_t* bb_dst, uint8_t* bs_dst,
                                          int x, const int* m0, const int* seg, int n0, uint64_t* bar) {
   asm volatile("// job %0" ::"n"(M));  // keeps the 16 cases of the switch apart
 #pragma unroll
   for (int h = 0; h < T3_SUB; ++h) tma_load_3d(a_dst + h * T3_TILE_A, &jobs.j[M].a, x, m0[h], seg[h], bar);
   tma_load_2d(bb_dst, &jobs.j[M].bb, x, n0, bar);
-  tma_load_2d(bs_dst, &jobs.j[M].bs, x, n0, bar);
+  if (!RAW) tma_load_2d(bs_dst, &jobs.j[M].bs, x, n0, bar);
 }
 
 // Epilogue of one tile of job M (the job's fields read at compile-time offsets
@@ -317,8 +350,10 @@ __device__ __forceinline__ void t3_epi_tile(const T3Jobs& jobs, int64_t tl, uint
   const int64_t ldy = J.ldy, y_seg_stride = J.y_seg_stride;
   float* const Y = J.Y;
   const float* const bias = J.bias;
-  const int64_t mp = tl / n_tiles_n;
-  const int n0 = (int)(tl % n_tiles_n) * TC_BN;
+  int64_t mp;
+  int nt;
+  t3_tile(tl, n_tiles_n, J.tri, mp, nt);
+  const int n0 = nt * TC_BN;
   const int tr = q * 32 + lane;  // row of the 128-row block
   const int half = lane >> 4, col = lane & 15;  // store phase: two rows of 16 columns per instruction
 #pragma unroll 1
@@ -353,6 +388,7 @@ __device__ __forceinline__ void t3_epi_tile(const T3Jobs& jobs, int64_t tl, uint
   }
 }
 
+template <bool RAW>
 __global__ void __launch_bounds__(T3J_THREADS, 1)
     gemm_tf32x3_tc_kernel(const __grid_constant__ T3Jobs jobs, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
@@ -415,8 +451,10 @@ __global__ void __launch_bounds__(T3J_THREADS, 1)
         const T3Fields& J = sj[jm];
         const int n_tiles_n = J.n_tiles_n, nk = J.nk, rb = J.rb, sbk = J.sb;
         const int64_t rb_per_seg = J.rb_per_seg;
-        const int64_t mp = tl / n_tiles_n;
-        const int n0 = (int)(tl % n_tiles_n) * TC_BN;
+        int64_t mp;
+        int nt;
+        t3_tile(tl, n_tiles_n, J.tri, mp, nt);
+        const int n0 = nt * TC_BN;
         int seg[T3_SUB], m0[T3_SUB];
 #pragma unroll
         for (int h = 0; h < T3_SUB; ++h) {  // first segment and row of each 128-row block (past the end: zero fill)
@@ -431,14 +469,14 @@ __global__ void __launch_bounds__(T3J_THREADS, 1)
             s_abort = 1;
             break;
           }
-          mbar_expect_tx(&full[s], T3_SUB * T3_TILE_A + 2 * T3_TILE_B);
+          mbar_expect_tx(&full[s], T3_SUB * T3_TILE_A + (RAW ? 1 : 2) * T3_TILE_B);
           uint8_t* const ad = sA + s * T3_SUB * T3_TILE_A;
           uint8_t* const bbd = sBb + s * T3_TILE_B;
           uint8_t* const bsd = sBs + s * T3_TILE_B;
           const int x = kb * T3_BK;
           switch (jm) {
 #define T3_CASE(M) \
-  case M: t3_issue<M>(jobs, ad, bbd, bsd, x, m0, seg, n0, &full[s]); break;
+  case M: t3_issue<M, RAW>(jobs, ad, bbd, bsd, x, m0, seg, n0, &full[s]); break;
             T3_CASE(0) T3_CASE(1) T3_CASE(2) T3_CASE(3) T3_CASE(4) T3_CASE(5) T3_CASE(6) T3_CASE(7)
             T3_CASE(8) T3_CASE(9) T3_CASE(10) T3_CASE(11) T3_CASE(12) T3_CASE(13) T3_CASE(14) T3_CASE(15)
 #undef T3_CASE
@@ -507,20 +545,12 @@ __global__ void __launch_bounds__(T3J_THREADS, 1)
         float4* src = reinterpret_cast<float4*>(sA + s * T3_SUB * T3_TILE_A);
         float4* dst = reinterpret_cast<float4*>(sAs + s * T3_SUB * T3_TILE_A);
 #pragma unroll 4
-        for (int j = 0; j < (int)(T3_SUB * T3_TILE_A / 16 / 128); ++j) {
-          const int idx = j * 128 + ct;
-          const float4 x = src[idx];
-          float4 b, sm;
-          b.x = tf32_rn(x.x);
-          b.y = tf32_rn(x.y);
-          b.z = tf32_rn(x.z);
-          b.w = tf32_rn(x.w);
-          sm.x = tf32_rn(x.x - b.x);
-          sm.y = tf32_rn(x.y - b.y);
-          sm.z = tf32_rn(x.z - b.z);
-          sm.w = tf32_rn(x.w - b.w);
-          src[idx] = b;
-          dst[idx] = sm;
+        for (int j = 0; j < (int)(T3_SUB * T3_TILE_A / 16 / 128); ++j) t3_split4(src + j * 128 + ct, dst + j * 128 + ct);
+        if (RAW) {
+          float4* bsrc = reinterpret_cast<float4*>(sBb + s * T3_TILE_B);
+          float4* bdst = reinterpret_cast<float4*>(sBs + s * T3_TILE_B);
+#pragma unroll 4
+          for (int j = 0; j < (int)(T3_TILE_B / 16 / 128); ++j) t3_split4(bsrc + j * 128 + ct, bdst + j * 128 + ct);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor cores
         __syncwarp();
@@ -855,12 +885,20 @@ cudaError_t split_tf32_t(const float* W, int rows, int cols, float* big, float* 
   return cudaGetLastError();
 }
 
+int64_t gemm_tf32x3_tiles(int64_t rows, int64_t cols, bool tri) {
+  const int64_t mp = (rows + T3_SUB * TC_BM - 1) / (T3_SUB * TC_BM), nt = (cols + TC_BN - 1) / TC_BN;
+  // the last row pair's column blocks end at the matrix
+  return tri ? (mp - 1) * mp + std::min<int64_t>(2 * mp, nt) : mp * nt;
+}
+
 cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* d, int n, unsigned int* status, cudaStream_t s) {
+  const bool raw = n > 0 && d[0].raw_w;
+  auto kern = raw ? gemm_tf32x3_tc_kernel<true> : gemm_tf32x3_tc_kernel<false>;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = t3_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(gemm_tf32x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   T3Jobs J;
   J.n = 0;
@@ -868,7 +906,7 @@ cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* d, int n, unsigned int* status,
   auto flush = [&]() -> cudaError_t {
     if (J.n == 0) return cudaSuccess;
     const int64_t grid = tiles < sms ? tiles : sms;
-    gemm_tf32x3_tc_kernel<<<(unsigned)grid, T3J_THREADS, smem, s>>>(J, status);
+    kern<<<(unsigned)grid, T3J_THREADS, smem, s>>>(J, status);
     J.n = 0;
     tiles = 0;
     return cudaGetLastError();
@@ -877,7 +915,8 @@ cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* d, int n, unsigned int* status,
     const T3JobDesc& q = d[i];
     if (q.seg_rows <= 0 || q.n_seg <= 0 || q.n_out <= 0) continue;
     if (q.K % 4 || q.ldx % 4 || q.ldw % 4 || q.x_seg_stride % 4 || (uintptr_t)q.X % 16 || (uintptr_t)q.Wbig % 16 ||
-        (uintptr_t)q.Wsmall % 16 || q.bias_period <= 0 || q.seg_rows > (int64_t)INT32_MAX ||
+        (uintptr_t)q.Wsmall % 16 || q.raw_w != raw || (q.tri && (q.n_seg != 1 || q.seg_rows != q.n_out)) ||
+        q.bias_period <= 0 || q.seg_rows > (int64_t)INT32_MAX ||
         q.n_seg > (int64_t)INT32_MAX)
       return cudaErrorInvalidValue;
     T3Job& j = J.j[J.n];
@@ -886,7 +925,7 @@ cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* d, int n, unsigned int* status,
     if (!make_map_seg_f32(&j.a, q.X, q.seg_rows, q.n_seg, q.K, q.ldx,
                           q.n_seg > 1 ? q.x_seg_stride : q.seg_rows * q.ldx, rb) ||
         !make_map(&j.bb, q.Wbig, q.n_out, q.K, q.ldw ? q.ldw : q.K, TC_BN, true) ||
-        !make_map(&j.bs, q.Wsmall, q.n_out, q.K, q.ldw ? q.ldw : q.K, TC_BN, true))
+        !make_map(&j.bs, raw ? q.Wbig : q.Wsmall, q.n_out, q.K, q.ldw ? q.ldw : q.K, TC_BN, true))
       return cudaErrorInvalidValue;
     j.f.bias = q.bias;
     j.f.Y = q.Y;
@@ -903,7 +942,8 @@ cudaError_t gemm_tf32x3_tc_jobs(const T3JobDesc* d, int n, unsigned int* status,
     j.f.n_tiles_n = (q.n_out + TC_BN - 1) / TC_BN;
     j.f.bias_period = q.bias_period;
     j.f.accumulate = q.accumulate ? 1 : 0;
-    tiles += ((j.f.n_mblk + T3_SUB - 1) / T3_SUB) * j.f.n_tiles_n;
+    j.f.tri = q.tri && rb == TC_BM ? 1 : 0;
+    tiles += j.f.tri ? gemm_tf32x3_tiles(q.seg_rows, q.n_out, true) : ((j.f.n_mblk + T3_SUB - 1) / T3_SUB) * j.f.n_tiles_n;
     j.f.tile_end = tiles;
     if (++J.n == kT3MaxJobs) {
       e = flush();

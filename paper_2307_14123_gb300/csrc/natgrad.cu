@@ -13,6 +13,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "det_util.cuh"
 #include "tc_ptx.cuh"
 
 namespace dq {
@@ -23,22 +24,71 @@ constexpr int64_t kNgChunk = 8192;  // K extent of one Gram chunk (FP32 accumula
 constexpr int kNgJobs = 16;         // chunks per GEMM launch
 constexpr int kNgRowWarps = 8;  // matvec: one warp per row of the Gram matrix
 
-// mean[p] = (1 / B) sum_b G[b][p], in FP64, one thread per column (fixed order over b)
-__global__ void ng_colmean_kernel(const float* __restrict__ G, int64_t B, int64_t P, double* __restrict__ mean) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  double s = 0;
-  for (int64_t b = 0; b < B; ++b) s += (double)G[b * P + p];
-  mean[p] = s / (double)B;
+// FP64 adds, multiply-adds and conversions from FP32 issue at 1.7 per clock and SM, 75 times slower
+// than FP32 ones: passes over G in FP64 were bound by them (one conversion, one operation per
+// element: 1.6 ms for 1024 x 412,656 gradients that memory delivers in 0.25 ms).  The sums below
+// (column means 1.62 -> 0.27 ms, centring 2.30 -> 0.48, the last product 1.60 -> 0.65)
+// are carried as three FP32 terms instead, hi + c1 + c2: every product and every addition into hi
+// and c1 keeps its rounding error exactly (TwoProd and TwoSum of Ogita, Rump, Oishi, "Accurate sum
+// and dot product", SIAM J. Sci. Comput. 26, 2005), so that only c2's additions round, at 2^-72 of
+// the sum: more than FP64 holds.
+struct Sum3 {
+  float hi, c1, c2;
+  __device__ __forceinline__ void add_c1(float e) {
+    const dfloat t = two_sum(c1, e);
+    c1 = t.hi;
+    c2 = __fadd_rn(c2, t.lo);
+  }
+  __device__ __forceinline__ void add(float x) {
+    const dfloat t = two_sum(hi, x);
+    hi = t.hi;
+    add_c1(t.lo);
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + ((double)c1 + (double)c2); }
+};
+
+// mean[p] = (1 / B) sum_b G[b][p] as an FP32 pair (to 2^-48).  A CTA sums 32 columns, warp g the
+// rows g, g + 8, ..; the warps' sums are added in FP64.
+__global__ void __launch_bounds__(kNgThreads)
+    ng_colmean_kernel(const float* __restrict__ G, int64_t B, int64_t P, float2* __restrict__ mean) {
+  __shared__ double sh[kNgThreads / 32][32];
+  const int lane = threadIdx.x % 32, g = threadIdx.x / 32;
+  const int64_t p = (int64_t)blockIdx.x * 32 + lane;
+  Sum3 s = {0.f, 0.f, 0.f};
+  if (p < P) {
+    const float* q = G + p;
+#pragma unroll 8
+    for (int64_t b = g; b < B; b += kNgThreads / 32) s.add(__ldg(q + b * P));
+  }
+  sh[g][lane] = s.value();
+  __syncthreads();
+  if (g == 0 && p < P) {
+    double t = 0;
+#pragma unroll
+    for (int k = 0; k < kNgThreads / 32; ++k) t += sh[k][lane];
+    t /= (double)B;
+    const float h = (float)t;
+    mean[p] = make_float2(h, (float)(t - (double)h));
+  }
 }
 
-// Gc[b][p] = G[b][p] - mean[p] with row pitch Pp (zeros in the padding)
-__global__ void ng_center_kernel(const float* __restrict__ G, const double* __restrict__ mean, int64_t B, int64_t P,
+// Gc[b][p] = G[b][p] - mean[p] (one rounding of the difference, up to 2^-20 of an ulp) with row
+// pitch Pp (zeros in the padding); a thread per column and 8 rows.
+constexpr int kNgCenterRows = 8;
+__global__ void ng_center_kernel(const float* __restrict__ G, const float2* __restrict__ mean, int64_t B, int64_t P,
                                  int64_t Pp, float* __restrict__ Gc) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= B * Pp) return;
-  const int64_t b = e / Pp, p = e - (e / Pp) * Pp;
-  Gc[e] = p < P ? (float)((double)G[b * P + p] - mean[p]) : 0.f;
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= Pp) return;
+  const float2 m = p < P ? mean[p] : make_float2(0.f, 0.f);
+  const int64_t b0 = (int64_t)blockIdx.y * kNgCenterRows;
+  float g[kNgCenterRows];
+#pragma unroll
+  for (int k = 0; k < kNgCenterRows; ++k) g[k] = p < P && b0 + k < B ? __ldg(G + (b0 + k) * P + p) : 0.f;
+#pragma unroll
+  for (int k = 0; k < kNgCenterRows; ++k) {
+    const dfloat d = two_sum(g[k], -m.x);
+    if (b0 + k < B) Gc[(b0 + k) * Pp + p] = __fadd_rn(d.hi, __fsub_rn(d.lo, m.y));
+  }
 }
 
 struct CgScalars {
@@ -124,14 +174,18 @@ __global__ void ng_cg_init_kernel(const float* __restrict__ w, int64_t B, const 
   }
 }
 
-// T (+)= sum of the chunks' Gram matrices, in FP64 and chunk order
-__global__ void ng_gram_add_kernel(const float* __restrict__ Tc, int n_chunks, int64_t BB, int first,
+// T (+)= sum of the chunks' Gram matrices, in FP64 and chunk order; mirror: only elements i >= j
+// are there, and stand for (j, i) as well
+__global__ void ng_gram_add_kernel(const float* __restrict__ Tc, int n_chunks, int64_t B, int first, int mirror,
                                    double* __restrict__ T) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, BB = B * B;
   if (e >= BB) return;
+  const int64_t i = e / B, j = e - (e / B) * B;
+  if (mirror && j > i) return;
   double s = first ? 0.0 : T[e];
   for (int c = 0; c < n_chunks; ++c) s += (double)Tc[(int64_t)c * BB + e];
   T[e] = s;
+  if (mirror) T[j * B + i] = s;
 }
 
 // T = (T + T^T) / 2: the 3 x TF32 products of T_ij and T_ji drop different low-order
@@ -231,8 +285,8 @@ __global__ void ng_cg_direction_kernel(int64_t B, const double* __restrict__ z, 
 // the systems that do not fit here: both give the same bits.
 // Against those (three launches per iteration, always max_iter of them; 17.4 +
 // 9.9 + 3.1 us each at B = 1024 until the residual is small) the call on 1024
-// walkers x 412,656 parameters takes 15.2 ms instead of 17.7, and a LiH training
-// step of 1024 walkers 8.0 ms instead of 10.7.
+// walkers x 412,656 parameters took 15.2 ms instead of 17.7, and a LiH training
+// step of 1024 walkers 8.0 ms instead of 10.7; 200 iterations at B = 1024 are 2.1 ms.
 // The barrier's wait is bounded; on a timeout every CTA leaves and
 // DQ_FLAG_TIMEOUT is set.
 // ---------------------------------------------------------------------------
@@ -271,7 +325,7 @@ __global__ void __launch_bounds__(kCgThreads, 1)
   double* p = reinterpret_cast<double*>(cg_smem);  // [B] direction
   double* r = p + B;                               // [B] residual
   double* dinv = r + B;                            // [B] 1 / diagonal
-  __shared__ double s_pap[kNgThreads], s_rr[kCgMaxGroups], s_rz[kCgMaxGroups];
+  __shared__ double s_pap[kNgThreads], s_rr[kCgMaxGroups], s_rz[kCgMaxGroups], s_scal[5];
   __shared__ int s_ok;
   const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
   const int row0 = blockIdx.x * rpc, row1 = min(B, row0 + rpc);
@@ -335,8 +389,17 @@ __global__ void __launch_bounds__(kCgThreads, 1)
       s_pap[tid] = s;
     }
     __syncthreads();
-    const double pAp = cg_tree256(s_pap, kNgThreads, lane);
-    const double alpha = pAp > 0 ? rz / pAp : 0.0;
+    // sums of sums and the scalars by one warp: an FP64 instruction holds the SM's pipe for 19 clocks
+    // whatever its lanes do, so that all 16 warps doing them cost 8 us per iteration
+    if (warp == 0) {
+      const double v = cg_tree256(s_pap, kNgThreads, lane);
+      if (lane == 0) {
+        s_scal[0] = v;
+        s_scal[1] = v > 0 ? rz / v : 0.0;
+      }
+    }
+    __syncthreads();
+    const double pAp = s_scal[0], alpha = s_scal[1];
     if (tid < row1 - row0) xi = fma(alpha, p[row0 + tid], xi);
     for (int g = warp; g < n_grp; g += kCgWarps) {  // r -= alpha A p; the group's r.r and r.z
       double vr[8], vz[8];
@@ -358,10 +421,18 @@ __global__ void __launch_bounds__(kCgThreads, 1)
       }
     }
     __syncthreads();
-    rr = cg_tree256(s_rr, n_grp, lane);
-    const double rz_new = cg_tree256(s_rz, n_grp, lane);
-    const double beta = rz > 0 ? rz_new / rz : 0.0;
-    rz = rz_new;
+    if (warp == 0) {
+      const double a = cg_tree256(s_rr, n_grp, lane), b = cg_tree256(s_rz, n_grp, lane);
+      if (lane == 0) {
+        s_scal[2] = a;
+        s_scal[3] = b;
+        s_scal[4] = rz > 0 ? b / rz : 0.0;
+      }
+    }
+    __syncthreads();
+    rr = s_scal[2];
+    rz = s_scal[3];
+    const double beta = s_scal[4];
     done = rr <= tol2 || it + 1 >= max_iter || !(pAp > 0);
     for (int i = tid; i < B; i += kCgThreads) p[i] = fma(beta, p[i], r[i] * dinv[i]);
     __syncthreads();
@@ -373,14 +444,46 @@ __global__ void __launch_bounds__(kCgThreads, 1)
   }
 }
 
-// delta[p] = sum_b x_b Gc[b][p] (fixed order over b); stats
-__global__ void ng_apply_kernel(const float* __restrict__ Gc, int64_t B, int64_t P, int64_t Pp,
-                                const double* __restrict__ x, float* __restrict__ delta) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= P) return;
-  double s = 0;
-  for (int64_t b = 0; b < B; ++b) s += x[b] * (double)Gc[b * Pp + q];
-  delta[q] = (float)s;
+// x as three FP32 terms (exact): the coefficients of ng_apply_kernel
+__global__ void ng_split_x_kernel(const double* __restrict__ x, int64_t B, float4* __restrict__ x3) {
+  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= B) return;
+  const float h = (float)x[b];
+  const double r1 = x[b] - (double)h;
+  const float l = (float)r1;
+  x3[b] = make_float4(h, l, (float)(r1 - (double)l), 0.f);
+}
+
+// delta[p] = sum_b x_b Gc[b][p] (fixed order): a CTA 32 columns, warp g the rows g, g + 8, ..
+__global__ void __launch_bounds__(kNgThreads)
+    ng_apply_kernel(const float* __restrict__ Gc, int64_t B, int64_t P, int64_t Pp, const float4* __restrict__ x3,
+                    float* __restrict__ delta) {
+  __shared__ double sh[kNgThreads / 32][32];
+  const int lane = threadIdx.x % 32, g = threadIdx.x / 32;
+  const int64_t q = (int64_t)blockIdx.x * 32 + lane;
+  Sum3 s = {0.f, 0.f, 0.f};
+  if (q < P) {
+#pragma unroll 8
+    for (int64_t b = g; b < B; b += kNgThreads / 32) {
+      const float v = __ldg(Gc + b * Pp + q);
+      const float4 c = __ldg(x3 + b);
+      const float p = __fmul_rn(c.x, v);
+      const float e = __fmaf_rn(c.x, v, -p);
+      const float p2 = __fmul_rn(c.y, v);
+      s.add(p);
+      s.add_c1(e);
+      s.add_c1(p2);
+      s.c2 = __fadd_rn(s.c2, __fmaf_rn(c.z, v, __fmaf_rn(c.y, v, -p2)));
+    }
+  }
+  sh[g][lane] = s.value();
+  __syncthreads();
+  if (g == 0 && q < P) {
+    double t = 0;
+#pragma unroll
+    for (int k = 0; k < kNgThreads / 32; ++k) t += sh[k][lane];
+    delta[q] = (float)t;
+  }
 }
 
 __global__ void ng_stats_kernel(const CgScalars* sc, double* stats) {
@@ -426,7 +529,7 @@ size_t natgrad_workspace(int64_t B, int64_t P) {
   const int64_t mv_ctas = (B + kNgRowWarps - 1) / kNgRowWarps;
   size_t o = 0;
   o += ng_align((size_t)P * 8);                 // mean
-  o += 3 * ng_align((size_t)B * Pp * 4);        // Gc, TF32 high, TF32 low
+  o += ng_align((size_t)B * Pp * 4);            // Gc
   o += ng_align((size_t)kNgJobs * B * B * 4);  // Gram matrices of the chunks of one launch
   o += ng_align((size_t)B * B * 8);             // Gram matrix (FP64)
   o += 5 * ng_align((size_t)B * 8);             // x, r, p, z, 1 / diag
@@ -434,6 +537,7 @@ size_t natgrad_workspace(int64_t B, int64_t P) {
   o += 2 * ng_align((size_t)(mv_ctas + 1024) * 8);  // partials
   o += ng_align(sizeof(CgScalars));
   o += ng_align(sizeof(unsigned int));          // arrivals at the solve's grid barrier
+  o += ng_align((size_t)B * 16);                // x in three FP32 terms
   return o;
 }
 
@@ -447,10 +551,8 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
     o += ng_align(bytes);
     return q;
   };
-  double* mean = reinterpret_cast<double*>(take((size_t)P * 8));
+  float2* mean = reinterpret_cast<float2*>(take((size_t)P * 8));
   float* Gc = reinterpret_cast<float*>(take((size_t)B * Pp * 4));
-  float* Wb = reinterpret_cast<float*>(take((size_t)B * Pp * 4));
-  float* Wsm = reinterpret_cast<float*>(take((size_t)B * Pp * 4));
   float* Tc = reinterpret_cast<float*>(take((size_t)kNgJobs * B * B * 4));
   double* T = reinterpret_cast<double*>(take((size_t)B * B * 8));
   double* x = reinterpret_cast<double*>(take((size_t)B * 8));
@@ -463,27 +565,52 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
   double* partials2 = reinterpret_cast<double*>(take((size_t)(mv_ctas + 1024) * 8));
   CgScalars* sc = reinterpret_cast<CgScalars*>(take(sizeof(CgScalars)));
   unsigned int* arrivals = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
+  float4* x3 = reinterpret_cast<float4*>(take((size_t)B * 16));
 
-  ng_colmean_kernel<<<ng_blocks(P, kNgThreads), kNgThreads, 0, s>>>(G, B, P, mean);
-  ng_center_kernel<<<ng_blocks(B * Pp, kNgThreads), kNgThreads, 0, s>>>(G, mean, B, P, Pp, Gc);
-  cudaError_t e = split_tf32(Gc, Wb, Wsm, B * Pp, s);
+  ng_colmean_kernel<<<ng_blocks(P, 32), kNgThreads, 0, s>>>(G, B, P, mean);
+  const dim3 cgrid(ng_blocks(Pp, kNgThreads), ng_blocks(B, kNgCenterRows));
+  ng_center_kernel<<<cgrid, kNgThreads, 0, s>>>(G, mean, B, P, Pp, Gc);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // T = Gc Gc^T (B x B): rows of Gc against the TF32 parts of Gc, in chunks of kNgChunk
-  // columns (each accumulated in FP32 on the tensor cores), the chunks added in FP64
+  // T = Gc Gc^T (B x B), in chunks of kNgChunk columns (each accumulated in FP32 on the tensor
+  // cores), the chunks added in FP64.  Both operands are split in shared memory.  Half the tiles
+  // (row >= column) and as many chunks per launch as leave the last wave of its tiles fullest:
+  // 1024 walkers have 32 tiles per chunk, 20 in the triangle; 51 chunks are 13 waves of 152 CTAs in
+  // launches of 16 chunks, 7 as triangles in launches of 15.  The triangle is taken where it saves
+  // a wave; where it does not (a few chunks fill one wave either way) both halves are computed and
+  // averaged.  (5.3 ms of launches with W split in memory first, 1.2 ms more, are 2.8 ms so.)
   const int64_t n_chunks = (Pp + kNgChunk - 1) / kNgChunk;
-  for (int64_t c0 = 0; c0 < n_chunks; c0 += kNgJobs) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  bool tri = false;
+  int per_launch = 0;
+  int64_t waves = 0;
+  for (int t = 0; t < 2; ++t) {
+    const int64_t tiles = gemm_tf32x3_tiles(B, B, t == 1);
+    for (int nj = kNgJobs; nj >= 1; --nj) {
+      const int64_t rest = n_chunks % nj;
+      const int64_t n = n_chunks / nj * ((nj * tiles + sms - 1) / sms) + (rest * tiles + sms - 1) / sms;
+      if (per_launch == 0 || n < waves) {
+        waves = n;
+        per_launch = nj;
+        tri = t == 1;
+      }
+    }
+  }
+  for (int64_t c0 = 0; c0 < n_chunks; c0 += per_launch) {
     T3JobDesc jd[kNgJobs];
     int nj = 0;
-    for (int64_t c = c0; c < n_chunks && nj < kNgJobs; ++c, ++nj) {
+    for (int64_t c = c0; c < n_chunks && nj < per_launch; ++c, ++nj) {
       const int64_t k0 = c * kNgChunk, kc = Pp - k0 < kNgChunk ? Pp - k0 : kNgChunk;
-      jd[nj] = T3JobDesc{Gc + k0, B, 1, 0, (int)kc, Pp, Wb + k0, Wsm + k0, (int)B, nullptr, 1,
-                         Tc + (int64_t)nj * B * B, B, 0, false, Pp};
+      jd[nj] = T3JobDesc{Gc + k0, B, 1, 0, (int)kc, Pp, Gc + k0, nullptr, (int)B, nullptr, 1,
+                         Tc + (int64_t)nj * B * B, B, 0, false, Pp, true, tri};
     }
     e = gemm_tf32x3_tc_jobs(jd, nj, status, s);
     if (e != cudaSuccess) return e;
-    ng_gram_add_kernel<<<ng_blocks(B * B, kNgThreads), kNgThreads, 0, s>>>(Tc, nj, B * B, c0 == 0 ? 1 : 0, T);
+    ng_gram_add_kernel<<<ng_blocks(B * B, kNgThreads), kNgThreads, 0, s>>>(Tc, nj, B, c0 == 0 ? 1 : 0, tri ? 1 : 0, T);
   }
-  ng_symmetrize_kernel<<<ng_blocks(B * B, kNgThreads), kNgThreads, 0, s>>>(T, B);
+  if (!tri) ng_symmetrize_kernel<<<ng_blocks(B * B, kNgThreads), kNgThreads, 0, s>>>(T, B);
   ng_cg_init_kernel<<<1, kNgThreads, 0, s>>>(w, B, T, x, r, p, dinv, sc, lam, tol, max_iter);
   if (!ng_solve(T, B, r, p, dinv, Ap, x, sc, arrivals, status, s, &e)) {
     // systems whose vectors do not fit one CTA's shared memory: three launches per iteration
@@ -495,7 +622,8 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
     }
   }
   if (e != cudaSuccess) return e;
-  ng_apply_kernel<<<ng_blocks(P, kNgThreads), kNgThreads, 0, s>>>(Gc, B, P, Pp, x, delta);
+  ng_split_x_kernel<<<ng_blocks(B, kNgThreads), kNgThreads, 0, s>>>(x, B, x3);
+  ng_apply_kernel<<<ng_blocks(P, 32), kNgThreads, 0, s>>>(Gc, B, P, Pp, x3, delta);
   if (stats) ng_stats_kernel<<<1, 1, 0, s>>>(sc, stats);
   return cudaGetLastError();
 }
