@@ -866,7 +866,22 @@ __global__ void __launch_bounds__(256, 2) messages_kernel_group(const __grid_con
 
 // Value-only messages (C = 1): one CTA per (walker, 32 features); a warp per
 // receiver, lanes over features; pair table and z of the walker staged in
-// shared memory, sender loops split by spin (no per-edge branch).
+// shared memory, sender loops split by spin (no per-edge branch).  The CTA's
+// slice of every filter row is staged as well (16-byte loads, all issued before
+// any is used): reading the filters where they are multiplied, twice per pair
+// and four at a time, was bound by latency: three layers of 4096 N2 walkers
+// 0.48 -> 0.35 ms.
+// Slices above kMvStage bytes (about 500 edges) are read in place: they would
+// leave too few CTAs per SM.
+constexpr size_t kMvStage = 64 * 1024;
+template <class T>
+inline size_t mv_tables(int N) {  // z and the pair table, padded to the filters' 16 bytes
+  return ((size_t)N * 32 * sizeof(T) + (size_t)N * N * sizeof(int) + 15) / 16 * 16;
+}
+template <class T>
+inline bool mv_staged(int E) {
+  return (size_t)E * 32 * sizeof(T) <= kMvStage;
+}
 template <class T, class TO>
 struct messages_value_kernel_args {
   const T* Z;
@@ -883,34 +898,57 @@ struct messages_value_kernel_args {
   int n_ee;
   int z_const;
   TO* msg;
+  int staged;
 };
 
 template <class T, class TO>
 __device__ __forceinline__ void messages_value_kernel_body(const int64_t bx_, const int by_, const int64_t nbx_, const T* __restrict__ Z, const T* __restrict__ z0, const T* __restrict__ ew,
                           const T* __restrict__ Y, const int* __restrict__ pair_of, int64_t Bc, int N, int n_up,
-                          int M, int D, int E, int n_ee, int z_const, TO* __restrict__ msg) {
+                          int M, int D, int E, int n_ee, int z_const, TO* __restrict__ msg, int staged) {
   extern __shared__ __align__(16) unsigned char mv_smem[];
   T* Zs = reinterpret_cast<T*>(mv_smem);           // [N][32]
   int* Ps = reinterpret_cast<int*>(Zs + N * 32);   // [N][N]
   const int64_t b = bx_;
   const int lane = threadIdx.x % 32, wq = threadIdx.x / 32, nw = blockDim.x / 32;
   const int d = by_ * 32 + lane;
+  const T* ewb = ew + b * E * D + d;  // this lane's feature of edge e at ewb[e * ldw]
+  int ldw = D;
+  if (staged) {
+    using V = typename Vec16<T>::type;
+    constexpr int VW = Vec16<T>::n, CH = 32 / VW, U = 4;  // 16-byte chunks per row; loads in flight per thread
+    const size_t off = ((size_t)N * 32 * sizeof(T) + (size_t)N * N * sizeof(int) + 15) / 16 * 16;
+    T* Ws = reinterpret_cast<T*>(mv_smem + off);   // [E][32]
+    const T* src = ew + b * E * D + by_ * 32;
+    for (int k0 = threadIdx.x; k0 < E * CH; k0 += U * blockDim.x) {
+      V v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * blockDim.x;
+        if (k < E * CH) v[u] = *reinterpret_cast<const V*>(src + (int64_t)(k / CH) * D + (k % CH) * VW);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * blockDim.x;
+        if (k < E * CH) *reinterpret_cast<V*>(Ws + k * VW) = v[u];
+      }
+    }
+    ewb = Ws + lane;
+    ldw = 32;
+  }
   for (int k = threadIdx.x; k < N * N; k += blockDim.x) Ps[k] = pair_of[k];
   for (int j = wq; j < N; j += nw)
-    Zs[j * 32 + lane] = d >= D ? T(0) : (z_const ? z0[(j < n_up ? 0 : D) + d] : Z[(b * N + j) * D + d]);
+    Zs[j * 32 + lane] = z_const ? z0[(j < n_up ? 0 : D) + d] : Z[(b * N + j) * D + d];
   __syncthreads();
-  if (d >= D) return;
-  const T* ewb = ew + b * E * D + d;
   for (int i = wq; i < N; i += nw) {
     const bool up = i < n_up;
     T su = 0, sd = 0, sn = 0;  // spin-up senders, spin-down senders, nuclei
 #pragma unroll 4
     for (int j = 0; j < n_up; ++j)
-      if (j != i) su += ewb[(int64_t)Ps[i * N + j] * D] * Zs[j * 32 + lane];
+      if (j != i) su += ewb[(int64_t)Ps[i * N + j] * ldw] * Zs[j * 32 + lane];
 #pragma unroll 4
     for (int j = n_up; j < N; ++j)
-      if (j != i) sd += ewb[(int64_t)Ps[i * N + j] * D] * Zs[j * 32 + lane];
-    for (int I = 0; I < M; ++I) sn += ewb[(int64_t)(n_ee + i * M + I) * D] * Y[(int64_t)I * D + d];
+      if (j != i) sd += ewb[(int64_t)Ps[i * N + j] * ldw] * Zs[j * 32 + lane];
+    for (int I = 0; I < M; ++I) sn += ewb[(int64_t)(n_ee + i * M + I) * ldw] * Y[(int64_t)I * D + d];
     const int n_same = up ? n_up : N - n_up, n_opp = N - n_same;
     TO* out = msg + (b * N + i) * 3 * D + d;
     out[0] = to_out((up ? su : sd) / T(n_same - 1 > 1 ? n_same - 1 : 1), out);
@@ -925,7 +963,7 @@ __global__ void __launch_bounds__(256) messages_value_kernel_group(const __grid_
   int64_t l_;
   const int m_ = grp_find(g, blockIdx.x, l_);
   const messages_value_kernel_args<T, TO>& a_ = g.a[m_];
-  messages_value_kernel_body<T, TO>(grp_bx(g, m_, l_), grp_by(g, m_, l_), g.nbx[m_], a_.Z, a_.z0, a_.ew, a_.Y, a_.pair_of, a_.Bc, a_.N, a_.n_up, a_.M, a_.D, a_.E, a_.n_ee, a_.z_const, a_.msg);
+  messages_value_kernel_body<T, TO>(grp_bx(g, m_, l_), grp_by(g, m_, l_), g.nbx[m_], a_.Z, a_.z0, a_.ew, a_.Y, a_.pair_of, a_.Bc, a_.N, a_.n_up, a_.M, a_.D, a_.E, a_.n_ee, a_.z_const, a_.msg, a_.staged);
 }
 
 // ---------------------------------------------------------------------------
@@ -2538,10 +2576,12 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
       const dq_handle_s& h = *m[k].h;
       const FwdDims& d = m[k].d;
       if (d.Bc <= 0) continue;
-      smem = std::max(smem, (size_t)d.N * 32 * sizeof(T) + (size_t)d.N * d.N * sizeof(int));
+      if (d.D % 32) return cudaErrorInvalidConfiguration;
+      const bool staged = mv_staged<T>(h.edges.n_all);
+      smem = std::max(smem, mv_tables<T>(d.N) + (staged ? (size_t)h.edges.n_all * 32 * sizeof(T) : 0));
       g.add({m[k].b.Z, m[k].b.z0, m[k].b.ew, m[k].params + h.off.layer[l].Y, h.d_pair_of, d.Bc, d.N, d.n_up, d.M, d.D,
-             h.edges.n_all, h.edges.n_ee, z_const && !h.el_init ? 1 : 0, out_of(m[k])},
-            d.Bc, (d.D + 31) / 32);
+             h.edges.n_all, h.edges.n_ee, z_const && !h.el_init ? 1 : 0, out_of(m[k]), staged ? 1 : 0},
+            d.Bc, d.D / 32);
     }
     if (g.n == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(messages_value_kernel_group<T, TO>,
