@@ -114,13 +114,17 @@ __global__ void geometry_kernel_group(const __grid_constant__ Grp<geometry_kerne
 
 // Edge hidden layer a = tanh(W1 e + b1) as a jet in d: (a, a', a'').
 // W1 and b1 of the three edge types are staged in shared memory once per CTA
-// ([t][q][a]); the persistent CTAs then stream blocks of kEdgesPerCta
-// consecutive (walker, edge) rows.  A thread computes kHiddenVec consecutive
-// features of one edge (vector loads of W1, vector stores), so D / kHiddenVec
-// threads cover an edge and one warp holds one edge type.
-constexpr int kEdgesPerCta = 32;
-constexpr int kHiddenThreads = 256;
-
+// ([t][q][a]); the persistent CTAs then stream blocks of epb consecutive
+// (walker, edge) rows, whose features arrive by asynchronous copies while the
+// previous block is computed (two buffers, one barrier per block).  A thread
+// computes kHiddenVec consecutive features of an edge (vector loads of W1,
+// vector stores), so D / kHiddenVec threads cover an edge and one warp holds one
+// edge type.  What bounds it beside the stores: shared-memory wavefronts.  So a
+// W1 load serves four edges of a type, and an edge's features are read a vector
+// at a time (1.75 wavefronts per edge and feature against 5 with edge pairs and
+// scalar reads).  Three layers of 4096 N2 walkers: 0.99 -> 0.82 ms with jets, 0.51 -> 0.40 values
+// only; FP64 (bound by tanh on the FP64 pipe, where the even spread of the blocks counts): twenty
+// layers of 512 LiH walkers 0.97 -> 0.59 ms.
 template <class T>
 struct Vec16;
 template <>
@@ -134,6 +138,11 @@ struct Vec16<double> {
   static constexpr int n = 2;
 };
 
+// Edges per block: 32, or 16 where 32 would leave an SM fewer than four blocks (a count of blocks
+// per SM that rounds up costs less then).
+constexpr int kEdgesPerBlk = 32;
+constexpr int kHiddenThreads = 256;
+
 template <class T>
 struct edge_hidden_kernel_args {
   const T* rbf;
@@ -144,7 +153,6 @@ struct edge_hidden_kernel_args {
   int n_ee;
   int D;
   int Q;
-  int ej;
   int64_t W1_0;
   int64_t W1_1;
   int64_t W1_2;
@@ -152,18 +160,35 @@ struct edge_hidden_kernel_args {
   int64_t b1_1;
   int64_t b1_2;
   T* eh;
+  int epb;
 };
 
-template <class T>
+// ej: 3 with jets, 1 for values only (a kernel of its own, with fewer registers)
+template <class T, int ej>
 __device__ __forceinline__ void edge_hidden_kernel_body(const int64_t bx_, const int by_, const int64_t nbx_, const T* __restrict__ rbf, const T* __restrict__ params, int64_t Bc, int E, int n_par,
-                       int n_ee, int D, int Q, int ej, int64_t W1_0, int64_t W1_1, int64_t W1_2, int64_t b1_0,
-                       int64_t b1_1, int64_t b1_2, T* __restrict__ eh) {
+                       int n_ee, int D, int Q, int64_t W1_0, int64_t W1_1, int64_t W1_2, int64_t b1_0,
+                       int64_t b1_1, int64_t b1_2, T* __restrict__ eh, int epb) {
   using V = typename Vec16<T>::type;
   constexpr int VW = Vec16<T>::n;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Ws = reinterpret_cast<T*>(smem_raw);  // [3][Q][D]
   T* bs = Ws + 3 * Q * D;                  // [3][D]
-  T* fs = bs + 3 * D;                      // [kEdgesPerCta][ej][Q] features of this block's rows
+  T* fs = bs + 3 * D;                      // [2][epb][ej][Q] features of a block's rows
+  const int64_t nrows = Bc * E;
+  const int rowlen = ej * Q;               // a multiple of 8
+  // the features of the block at row be0 into a buffer (consecutive rows: one contiguous range)
+  auto issue = [&](int64_t be0, T* dst) {
+    if (be0 < nrows) {
+      const int n = (int)min((int64_t)epb, nrows - be0) * rowlen / VW;
+      const T* src = rbf + be0 * rowlen;
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+      for (int k = threadIdx.x; k < n; k += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + k * 16), "l"(src + k * VW) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int64_t step = (int64_t)nbx_ * epb;
+  issue((int64_t)bx_ * epb, fs);
   const int64_t W1o[3] = {W1_0, W1_1, W1_2}, b1o[3] = {b1_0, b1_1, b1_2};
   for (int t = 0; t < 3; ++t)
     for (int a = threadIdx.x; a < D; a += blockDim.x) {
@@ -174,12 +199,13 @@ __device__ __forceinline__ void edge_hidden_kernel_body(const int64_t bx_, const
   const int tpe = D / VW;                        // threads per edge
   const int epp = blockDim.x / tpe;              // edges in parallel
   const int er = threadIdx.x / tpe, a0 = (threadIdx.x % tpe) * VW;
-  const int64_t nrows = Bc * E;
-  for (int64_t be0 = (int64_t)bx_ * kEdgesPerCta; be0 < nrows; be0 += (int64_t)nbx_ * kEdgesPerCta) {
-    const int nb = (int)min((int64_t)kEdgesPerCta, nrows - be0);
-    __syncthreads();  // previous block's features consumed (and the weights staged)
-    for (int k = threadIdx.x; k < nb * ej * Q; k += blockDim.x) fs[k] = rbf[be0 * ej * Q + k];
-    __syncthreads();
+  int buf = 0;
+  for (int64_t be0 = (int64_t)bx_ * epb; be0 < nrows; be0 += step, buf ^= 1) {
+    const int nb = (int)min((int64_t)epb, nrows - be0);
+    const T* fb = fs + buf * epb * rowlen;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this block's features (and the weights) staged; the other buffer is consumed
+    issue(be0 + step, fs + (buf ^ 1) * epb * rowlen);
     if (er >= epp) continue;
     auto type_of = [&](int r) {
       const int e = (int)((be0 + r) % E);
@@ -201,22 +227,33 @@ __device__ __forceinline__ void edge_hidden_kernel_body(const int64_t bx_, const
           h1[n][v] = 0;
           h2[n][v] = 0;
         }
-#pragma unroll 4
-      for (int q = 0; q < Q; ++q) {
-        const V wv = *reinterpret_cast<const V*>(W + q * D);
-        const T* w = reinterpret_cast<const T*>(&wv);
+#pragma unroll 1
+      for (int q0 = 0; q0 < Q; q0 += VW) {
+        V wv[VW];
+#pragma unroll
+        for (int k = 0; k < VW; ++k) wv[k] = *reinterpret_cast<const V*>(W + (q0 + k) * D);
 #pragma unroll
         for (int n = 0; n < NE; ++n) {
-          const T* f = fs + (r + n) * ej * Q;
-          const T f0 = f[q];
-#pragma unroll
-          for (int v = 0; v < VW; ++v) h[n][v] += w[v] * f0;
+          const T* f = fb + (r + n) * rowlen + q0;
+          const V f0v = *reinterpret_cast<const V*>(f);
+          V f1v = f0v, f2v = f0v;
           if (ej == 3) {
-            const T f1 = f[Q + q], f2 = f[2 * Q + q];
+            f1v = *reinterpret_cast<const V*>(f + Q);
+            f2v = *reinterpret_cast<const V*>(f + 2 * Q);
+          }
 #pragma unroll
-            for (int v = 0; v < VW; ++v) {
-              h1[n][v] += w[v] * f1;
-              h2[n][v] += w[v] * f2;
+          for (int k = 0; k < VW; ++k) {
+            const T* w = reinterpret_cast<const T*>(&wv[k]);
+            const T f0 = reinterpret_cast<const T*>(&f0v)[k];
+#pragma unroll
+            for (int v = 0; v < VW; ++v) h[n][v] += w[v] * f0;
+            if (ej == 3) {
+              const T f1 = reinterpret_cast<const T*>(&f1v)[k], f2 = reinterpret_cast<const T*>(&f2v)[k];
+#pragma unroll
+              for (int v = 0; v < VW; ++v) {
+                h1[n][v] += w[v] * f1;
+                h2[n][v] += w[v] * f2;
+              }
             }
           }
         }
@@ -251,7 +288,7 @@ __device__ __forceinline__ void edge_hidden_kernel_body(const int64_t bx_, const
         if (r + 1 < nb) rows(std::integral_constant<int, 1>{}, r + 1);
       }
     };
-    if (ej == 1) {  // value rows: four edges per W1 load (registers allow it)
+    if (4 * epp <= epb) {  // four edges per W1 load where the block has four for every group of threads
       for (int r = 4 * er; r < nb; r += 4 * epp) {
         const int t = type_of(r);
         if (r + 3 < nb && type_of(r + 1) == t && type_of(r + 2) == t && type_of(r + 3) == t) {
@@ -261,19 +298,22 @@ __device__ __forceinline__ void edge_hidden_kernel_body(const int64_t bx_, const
           if (r + 2 < nb) pair(r + 2);
         }
       }
-    } else {
+    } else if (2 * epp <= epb) {
       for (int r = 2 * er; r < nb; r += 2 * epp) pair(r);
+    } else {
+      for (int r = er; r < nb; r += epp) rows(std::integral_constant<int, 1>{}, r);
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // One launch over several molecules: block b runs entry m of the table.
-template <class T>
+template <class T, int ej>
 __global__ void __launch_bounds__(kHiddenThreads) edge_hidden_kernel_group(const __grid_constant__ Grp<edge_hidden_kernel_args<T>> g) {
   int64_t l_;
   const int m_ = grp_find(g, blockIdx.x, l_);
   GRP_STATIC(m_, const auto& a_ = g.a[K_];
-             edge_hidden_kernel_body<T>(grp_bx(g, K_, l_), grp_by(g, K_, l_), g.nbx[K_], a_.rbf, a_.params, a_.Bc, a_.E, a_.n_par, a_.n_ee, a_.D, a_.Q, a_.ej, a_.W1_0, a_.W1_1, a_.W1_2, a_.b1_0, a_.b1_1, a_.b1_2, a_.eh);)
+             edge_hidden_kernel_body<T, ej>(grp_bx(g, K_, l_), grp_by(g, K_, l_), g.nbx[K_], a_.rbf, a_.params, a_.Bc, a_.E, a_.n_par, a_.n_ee, a_.D, a_.Q, a_.W1_0, a_.W1_1, a_.W1_2, a_.b1_0, a_.b1_1, a_.b1_2, a_.eh, a_.epb);)
 }
 
 // ---------------------------------------------------------------------------
@@ -2475,19 +2515,20 @@ cudaError_t launch_edge_hidden_group(const MolFwd<T>* m, int n, int l, cudaStrea
     const int ej = d.C > 1 ? 3 : 1;
     const auto& y = h.off.layer[l];
     const int64_t rows = d.Bc * h.edges.n_all;
-    smem = std::max(smem, ((size_t)3 * d.Q * d.D + 3 * d.D + (size_t)kEdgesPerCta * ej * d.Q) * sizeof(T));
-    const int64_t nblk = (rows + kEdgesPerCta - 1) / kEdgesPerCta;
+    const int epb = rows_all < (int64_t)4 * kEdgesPerBlk * device_sms() ? kEdgesPerBlk / 2 : kEdgesPerBlk;
+    smem = std::max(smem, ((size_t)3 * d.Q * d.D + 3 * d.D + (size_t)2 * epb * ej * d.Q) * sizeof(T));
+    const int64_t nblk = (rows + epb - 1) / epb;
     int64_t share = (grid_all * rows + rows_all - 1) / rows_all;
     share = std::max<int64_t>(1, std::min(share, nblk));
-    g.add({m[k].b.rbf, m[k].params, d.Bc, h.edges.n_all, h.edges.n_par, h.edges.n_ee, d.D, d.Q, ej, y.W1[0], y.W1[1],
-           y.W1[2], y.b1[0], y.b1[1], y.b1[2], m[k].b.eh},
+    g.add({m[k].b.rbf, m[k].params, d.Bc, h.edges.n_all, h.edges.n_par, h.edges.n_ee, d.D, d.Q, y.W1[0], y.W1[1],
+           y.W1[2], y.b1[0], y.b1[1], y.b1[2], m[k].b.eh, epb},
           share);
   }
   if (g.n == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(edge_hidden_kernel_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  auto kern = m[0].d.C > 1 ? edge_hidden_kernel_group<T, 3> : edge_hidden_kernel_group<T, 1>;  // all entries alike
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  edge_hidden_kernel_group<T><<<(unsigned)g.blocks(), kHiddenThreads, smem, s>>>(g);
+  kern<<<(unsigned)g.blocks(), kHiddenThreads, smem, s>>>(g);
   return cudaGetLastError();
 }
 
