@@ -284,6 +284,8 @@ inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
     if (e_ != cudaSuccess) return DQ_ERR_CUDA;          \
   } while (0)
 
+inline RowMap rm(int64_t ld) { return RowMap{1, ld, 0}; }
+
 template <class T>
 dq_status run_forward(const dq_handle_s& h, const T* params, const T* r, int64_t B, bool jets, T* logabs,
                       int8_t* sign, T* e_loc, unsigned char* ws, size_t ws_bytes, cudaStream_t s,
@@ -342,6 +344,7 @@ dq_status run_forward(const dq_handle_s& h, const T* params, const T* r, int64_t
   for (int64_t b0 = 0; b0 < B; b0 += Bmax) {
     const int64_t nb = std::min<int64_t>(Bmax, B - b0);
     const FwdDims d{nb, N, h.n_up, h.n_dn, h.M, D, K, h.Q, C};
+    place_split(bf, d, split_messages(d) && !use_fused(h, jets));
     DQ_LAUNCH(h, kb + PK_GEOMETRY, launch_geometry<T>(h, d, r + b0 * N * 3, bf, s));
     // embeddings of the electron-nucleus difference vectors (Eq. 13, second case): layer 0 then
     // takes the general path below instead of the spin-embedding shortcut
@@ -411,20 +414,37 @@ dq_status run_forward(const dq_handle_s& h, const T* params, const T* r, int64_t
         }
         DQ_LAUNCH(h, kb + PK_MESSAGES, launch_messages<T>(h, d, params, l, false, bf, s));
       }
-      const RowMap mrow{(int64_t)N * C, (int64_t)N * C * 3 * D, 3 * D};
-      if (use_tc) {
-        DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_bf16_tc(bf.msg_bf, rows, 3 * D, 3 * D, wg_bf(l), D,
-                                                       reinterpret_cast<const float*>(params + y.b_g), C,
-                                                       reinterpret_cast<float*>(bf.Z), D, h.d_status, s));
-      } else if (use_t3) {
-        DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_tf32x3_tc(reinterpret_cast<const float*>(bf.msg), rows, 3 * D, 3 * D,
-                                                         wg_t3(l, 0), wg_t3(l, 1), D,
-                                                         reinterpret_cast<const float*>(params + y.b_g), C,
-                                                         reinterpret_cast<float*>(bf.Z), D, h.d_status, s));
-      } else {
-        DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_nt<T>(bf.msg, mrow, params + y.W_g, params + y.b_g, C, bf.Z, node, rows,
-                                                     D, 3 * D, false, s));
+      // update map W_g [m_par; m_anti; m_nuc] + b_g: all rows, or (split messages) the
+      // electron-electron blocks of all rows and the five special rows per electron apart
+      struct Map {
+        const void* X;
+        int64_t rows;
+        int K, bias_period;
+        T* Y;
+      };
+      const void* msg = use_tc ? bf.msg_bf : bf.msg;
+      const Map maps[2] = {{msg, rows, (bf.msg5 ? 2 : 3) * D, bf.msg5 ? 0 : C, bf.Z},
+                           {bf.msg5, nb * N * 5, 3 * D, 5, bf.un5}};
+      T3JobDesc jd[2];
+      int nj = 0;
+      for (int q = 0; q < (bf.msg5 ? 2 : 1); ++q) {
+        const Map& mq = maps[q];
+        const T* bg = mq.bias_period ? params + y.b_g : nullptr;
+        const int period = std::max(1, mq.bias_period);
+        if (use_tc) {
+          DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_bf16_tc(mq.X, mq.rows, mq.K, mq.K, wg_bf(l), D,
+                                                         reinterpret_cast<const float*>(bg), period,
+                                                         reinterpret_cast<float*>(mq.Y), D, h.d_status, s, 3 * D));
+        } else if (use_t3) {
+          jd[nj++] = T3JobDesc{static_cast<const float*>(mq.X), mq.rows, 1, 0, mq.K, mq.K, wg_t3(l, 0), wg_t3(l, 1), D,
+                               reinterpret_cast<const float*>(bg), period, reinterpret_cast<float*>(mq.Y), D, 0, false,
+                               3 * D};
+        } else {
+          DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_nt<T>(static_cast<const T*>(mq.X), rm(mq.K), params + y.W_g, bg, period,
+                                                       mq.Y, rm(D), mq.rows, D, mq.K, false, s, 3 * D));
+        }
       }
+      if (nj > 0) DQ_LAUNCH(h, kb + PK_GEMM_UPDATE, gemm_tf32x3_tc_jobs(jd, nj, h.d_status, s));
       DQ_LAUNCH(h, kb + PK_UPDATE, launch_update<T>(h, d, params, l == 0 && !h.el_init, bf, s));
     }
     const int ns[2] = {h.n_up, h.n_dn}, i0[2] = {0, h.n_up};
@@ -534,7 +554,6 @@ GradPlan plan_grad(const dq_handle_s& h, int64_t Bc, size_t elem) {
   return p;
 }
 
-inline RowMap rm(int64_t ld) { return RowMap{1, ld, 0}; }
 
 template <class T>
 dq_status run_grad(const dq_handle_s& h, const T* params, const T* r, int64_t B, const T* weights, int mode, T* G,
@@ -1072,6 +1091,7 @@ dq_status run_forward_multi(const dq_multi_s& g, const T* const* params, const T
         rest[m] = mf[m];
         fused[m] = use_fused(*g.h[m], jets) && mf[m].d.Bc > 0;
         if (fused[m]) rest[m].d.Bc = 0;
+        place_split(rest[m].b, rest[m].d, split_messages(rest[m].d) && rest[m].d.Bc > 0);
       }
       DQ_LAUNCH(H, kb + PK_MESSAGES, launch_messages_group<T>(rest, n, l, l == 0, s));
       nj = 0;
@@ -1079,16 +1099,23 @@ dq_status run_forward_multi(const dq_multi_s& g, const T* const* params, const T
         const dq_handle_s& h = *g.h[m];
         const FwdDims& d = rest[m].d;
         if (d.Bc <= 0) continue;
-        const int64_t rows = d.Bc * d.N * d.C;
+        const FwdBuffers<T>& rb = rest[m].b;
+        const int64_t rows[2] = {d.Bc * d.N * d.C, d.Bc * d.N * 5};
+        const bool split = rb.msg5 != nullptr;  // (as in run_forward)
         const float* bg = reinterpret_cast<const float*>(params[m] + h.off.layer[l].b_g);
-        if (use_tc) {
-          DQ_LAUNCH(H, kb + PK_GEMM_UPDATE,
-                    gemm_bf16_tc(mf[m].b.msg_bf, rows, 3 * h.D, 3 * h.D, Wbf[m] + (size_t)l * 4 * h.D * h.D * 2, h.D,
-                                 bg, d.C, reinterpret_cast<float*>(mf[m].b.Z), h.D, H.d_status, s));
-        } else {
-          jd[nj++] = T3JobDesc{reinterpret_cast<const float*>(mf[m].b.msg), rows, 1, 0, 3 * h.D, 3 * h.D,
-                               w3[m].wg(l, 0), w3[m].wg(l, 1), h.D, bg, d.C, reinterpret_cast<float*>(mf[m].b.Z), h.D,
-                               0, false};
+        for (int q = 0; q < (split ? 2 : 1); ++q) {
+          const void* X = q == 1 ? rb.msg5 : use_tc ? rb.msg_bf : rb.msg;
+          const int Kq = split && q == 0 ? 2 * h.D : 3 * h.D;
+          const float* bq = split && q == 0 ? nullptr : bg;
+          const int period = q == 1 ? 5 : d.C;
+          float* Y = reinterpret_cast<float*>(q == 1 ? rb.un5 : rb.Z);
+          if (use_tc) {
+            DQ_LAUNCH(H, kb + PK_GEMM_UPDATE, gemm_bf16_tc(X, rows[q], Kq, Kq, Wbf[m] + (size_t)l * 4 * h.D * h.D * 2, h.D,
+                                                           bq, period, Y, h.D, H.d_status, s, 3 * h.D));
+          } else {
+            jd[nj++] = T3JobDesc{static_cast<const float*>(X), rows[q], 1, 0, Kq, Kq, w3[m].wg(l, 0), w3[m].wg(l, 1), h.D,
+                                 bq, period, Y, h.D, 0, false, 3 * h.D};
+          }
         }
       }
       if (!use_tc) DQ_LAUNCH(H, kb + PK_GEMM_UPDATE, gemm_tf32x3_tc_jobs(jd, nj, H.d_status, s));
@@ -1102,6 +1129,7 @@ dq_status run_forward_multi(const dq_multi_s& g, const T* const* params, const T
                                        mf[m].b.geo, mf[m].b.msg, w3[m].wg(l, 0), w3[m].wg(l, 1),
                                        use_tc ? Wbf[m] + (size_t)l * 4 * h.D * h.D * 2 : nullptr, s));
           FwdBuffers<T> bu = mf[m].b;
+          place_split(bu, mf[m].d, false);
           bu.F_bf = nullptr;
           DQ_LAUNCH(H, kb + PK_UPDATE, launch_update<T>(h, mf[m].d, params[m], z_const, bu, s));
         }

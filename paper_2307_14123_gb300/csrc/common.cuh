@@ -193,15 +193,15 @@ struct RowMap {
 };
 
 // Y[r][n] (+)= sum_k X[r][k] W[n][k] + (r % bias_period == 0 ? bias[n] : 0).
-// W is [n_out][K] row-major.  K % 8 == 0; X and Y rows 16-byte aligned.
+// W is [n_out][K] row-major with row pitch ldw (0: K).  K % 8 == 0; X and Y rows 16-byte aligned.
 template <class T>
 cudaError_t gemm_nt(const T* X, RowMap mx, const T* W, const T* bias, int bias_period, T* Y, RowMap my,
-                    int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s);
+                    int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s, int ldw = 0);
 
 // BF16 tensor-core GEMM (gemm_tc.cu): Y[r][n] = X[r][:] . W[n][:] (+ bias on
-// rows r % bias_period == 0); X, W BF16 K-major, Y FP32.
+// rows r % bias_period == 0); X, W BF16 K-major (W's row pitch ldw, 0: K), Y FP32.
 cudaError_t gemm_bf16_tc(const void* X, int64_t rows, int K, int64_t ldx, const void* W, int n_out, const float* bias,
-                         int bias_period, float* Y, int64_t ldy, unsigned int* status, cudaStream_t s);
+                         int bias_period, float* Y, int64_t ldy, unsigned int* status, cudaStream_t s, int64_t ldw = 0);
 
 // FP32-accurate tensor-core GEMM (3 x TF32 split, gemm_tc.cu): X FP32 [rows][K]
 // (K % 4 == 0), W pre-split by split_tf32 into TF32 big and small parts.
@@ -303,7 +303,28 @@ struct FwdBuffers {
   // BF16 mode only (nullptr otherwise): GEMM inputs of the embedding layers
   void* msg_bf;  // [Bc][N][C][3D]  messages, BF16 (replaces msg)
   void* F_bf;    // [Bc][N][C][D]   BF16 copy of the embeddings
+  // Split messages (jets of the separate layer kernels, split_messages): the electron-nucleus
+  // messages are zero but on five channels per electron (value, own coordinates, Laplacian: d_iI
+  // depends on r_i alone), so msg / msg_bf holds [Bc][N][C][2D] without them, and the five channels'
+  // whole rows stand apart, with their own update-map products.
+  void* msg5;  // [Bc][N][5][3D]  same type as the messages; nullptr: not split
+  T* un5;      // [Bc][N][5][D]   W_g msg5 + b_g
 };
+// Where the split pays: the update map reads 2 C + 15 instead of 3 C blocks per electron, for two
+// more launches.  C = 3 N + 2 >= 29 saves 15 % and more of the map and of the message traffic; both
+// parts fit the unsplit buffer from C = 25 on.
+inline bool split_messages(const FwdDims& d) { return d.C > 1 && d.N >= 9; }
+// Places a chunk's split messages in the buffers of the unsplit ones.
+template <class T>
+void place_split(FwdBuffers<T>& b, const FwdDims& d, bool split) {
+  b.msg5 = nullptr;
+  b.un5 = nullptr;
+  if (!split) return;
+  const int64_t el = b.msg_bf ? 2 : (int64_t)sizeof(T), bn = d.Bc * d.N;
+  unsigned char* base = b.msg_bf ? static_cast<unsigned char*>(b.msg_bf) : reinterpret_cast<unsigned char*>(b.msg);
+  b.msg5 = base + bn * d.C * 2 * d.D * el;
+  b.un5 = reinterpret_cast<T*>(static_cast<unsigned char*>(b.msg5) + bn * 15 * d.D * el);
+}
 
 // Grouped sampler and reduction launches (mcmc.cu), one entry per molecule.
 template <class T>
@@ -367,11 +388,11 @@ bool layer_fused_supported(const dq_handle_s& h);
 // Jet messages of molecules past the fused layer kernel (messages_large.cu): FP32 modes, node
 // channels from the node map (not the spin-embedding constants), 3 N + 2 channels, D a multiple
 // of 32, N <= 48 with at most 24 electrons per spin.  Writes all three message slots of msg
-// ([Bc][N][C][3D], FP32, or BF16 when bf16_out).
+// ([Bc][N][C][3D], FP32, or BF16 when bf16_out), or, with msg5, the split form of FwdBuffers.
 bool messages_large_supported(const dq_handle_s& h, const FwdDims& d);
 cudaError_t launch_messages_large(const dq_handle_s& h, const FwdDims& d, const float* params, int l,
-                                  const float* Z, const float* ew, const float* geo, void* msg, bool bf16_out,
-                                  cudaStream_t s);
+                                  const float* Z, const float* ew, const float* geo, void* msg, void* msg5,
+                                  bool bf16_out, cudaStream_t s);
 cudaError_t launch_layer_fused(const dq_handle_s& h, const FwdDims& d, const float* params, int l, bool z_const,
                                float* Z, const float* z0, const float* ew, const float* geo, float* mn,
                                const float* wg_hi, const float* wg_lo, const void* wg_bf, cudaStream_t s);

@@ -589,13 +589,14 @@ struct messages_kernel_args {
   int z_const;
   int stage_w1;
   TO* msg;
+  TO* msg5;  // the split form of FwdBuffers (nullptr: not split)
 };
 
 template <class T, class TO, int IB, int CB, int L>
 __device__ __forceinline__ void messages_kernel_body(const int64_t bx_, const int by_, const int64_t nbx_, const T* __restrict__ Z, const T* __restrict__ z0, const T* __restrict__ ew,
                     const T* __restrict__ geo, const T* __restrict__ Y, const int* __restrict__ pair_of, int N,
                     int n_up, int M, int C, int D, int E, int n_ee, int z_const, int stage_w1,
-                    TO* __restrict__ msg) {
+                    TO* __restrict__ msg, TO* __restrict__ msg5) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int ej = 3;
   const MsgSmem lay = msg_smem_layout<T>(N, IB, CB, stage_w1 != 0, L);
@@ -648,10 +649,12 @@ __device__ __forceinline__ void messages_kernel_body(const int64_t bx_, const in
     Id[k] = id;
   }
   for (int k = tid; k < IB * N * 3; k += blockDim.x) Us[NN * 3 + k] = T(0);
-  TO* mb = msg + b * N * C * 3 * D + d0 + lane;
+  const int mp = (msg5 ? 2 : 3) * D;  // row pitch of msg
+  TO* mb = msg + b * N * C * mp + d0 + lane;
+  TO* m5 = msg5 ? msg5 + b * N * 15 * D + d0 + lane : nullptr;
   // electron-nucleus part of every output: zero except in the value, Laplacian and
-  // own-coordinate channels, which are written after phase 1
-  for (int i = grp; i < N; i += ngroups) {
+  // own-coordinate channels, which are written after phase 1 (split: nowhere else)
+  for (int i = grp; i < N && m5 == nullptr; i += ngroups) {
     TO* o = mb + (int64_t)i * C * 3 * D + 2 * D;
     for (int c = 0; c < C; ++c, o += 3 * D) *o = to_out(T(0), o);
   }
@@ -764,7 +767,8 @@ __device__ __forceinline__ void messages_kernel_body(const int64_t bx_, const in
     const int c = kind == 0 ? 0 : (kind == 1 ? C - 1 : 1 + 3 * i + (kind - 2));
     const T v = kind == 0 ? SPd[i * L + lane]
                           : (kind == 1 ? SPc[(i * 3 + 2) * L + lane] : SPb[((i * 3 + kind - 2) * 3 + 2) * L + lane]);
-    TO* o = mb + ((int64_t)i * C + c) * 3 * D + 2 * D;
+    const int slot = kind == 0 ? 0 : kind == 1 ? 4 : kind - 1;
+    TO* o = (m5 ? m5 + ((int64_t)i * 5 + slot) * 3 * D : mb + ((int64_t)i * C + c) * 3 * D) + 2 * D;
     *o = to_out(v * nuM, o);
   }
 
@@ -872,14 +876,18 @@ __device__ __forceinline__ void messages_kernel_body(const int64_t bx_, const in
         }
       }
       const T nu = T(1) / T(pass == 0 ? (sbn - 1 > 1 ? sbn - 1 : 1) : (osn > 1 ? osn : 1));
-      TO* ob = mb + ((int64_t)i0 * C + c0) * 3 * D + pass * D;
+      TO* ob = mb + ((int64_t)i0 * C + c0) * mp + pass * D;
 #pragma unroll
       for (int a = 0; a < IB; ++a) {
         if (a >= ni) continue;
 #pragma unroll
         for (int q = 0; q < CB; ++q) {
           if (q >= nc) continue;
-          TO* o = ob + ((int64_t)a * C + q) * 3 * D;
+          TO* o = ob + ((int64_t)a * C + q) * mp;
+          if (m5) {
+            const int slot = c0 + q == 0 ? 0 : q == qlap ? 4 : eq[q] == i0 + a ? 1 + xq[q] : -1;
+            if (slot >= 0) o = m5 + ((int64_t)(i0 + a) * 5 + slot) * 3 * D + pass * D;
+          }
           *o = to_out(acc[a][q] * nu, o);
         }
       }
@@ -897,11 +905,11 @@ __global__ void __launch_bounds__(256, 2) messages_kernel_group(const __grid_con
   if (g.tag[m_] == 16)
     messages_kernel_body<T, TO, IB, CB, 16>(grp_bx(g, m_, l_), grp_by(g, m_, l_), g.nbx[m_], a_.Z, a_.z0, a_.ew, a_.geo,
                                             a_.Y, a_.pair_of, a_.N, a_.n_up, a_.M, a_.C, a_.D, a_.E, a_.n_ee,
-                                            a_.z_const, a_.stage_w1, a_.msg);
+                                            a_.z_const, a_.stage_w1, a_.msg, a_.msg5);
   else
     messages_kernel_body<T, TO, IB, CB, kMsgLanes>(grp_bx(g, m_, l_), grp_by(g, m_, l_), g.nbx[m_], a_.Z, a_.z0, a_.ew,
                                                    a_.geo, a_.Y, a_.pair_of, a_.N, a_.n_up, a_.M, a_.C, a_.D, a_.E,
-                                                   a_.n_ee, a_.z_const, a_.stage_w1, a_.msg);
+                                                   a_.n_ee, a_.z_const, a_.stage_w1, a_.msg, a_.msg5);
 }
 
 // Value-only messages (C = 1): one CTA per (walker, 32 features); a warp per
@@ -1022,44 +1030,119 @@ struct update_kernel_args {
   int D;
   int from_spin;
   __nv_bfloat16* Fbf;
+  const T* P5;
 };
 
+// A thread owns one 16-byte vector of features of one electron and walks its channels in batches:
+// every load of a batch (pre-activations and embeddings) is issued before any store, which the
+// compiler may not do by itself because the embeddings are updated in place.  The kernel is bound
+// by HBM; a feature per thread and one channel at a time kept too few bytes in flight: three
+// layers of 4096 N2 walkers 2.14 -> 1.49 ms, four of 1024 C4H4 walkers with BF16 copies 9.75 -> 4.78.
+// P5 (nullable): the pre-activations of an electron's value, own-coordinate and Laplacian channels
+// [b][i][5][D], instead of those rows of P.
+constexpr int kUpdBatch = 4;
 template <class T>
 __device__ __forceinline__ void update_kernel_body(const int64_t bx_, const int by_, const int64_t nbx_, const T* __restrict__ P, const T* Fin, T* Fout, const T* __restrict__ E_spin,
                               int64_t Bc, int N, int n_up, int C, int D, int from_spin,
-                              __nv_bfloat16* __restrict__ Fbf) {
+                              __nv_bfloat16* __restrict__ Fbf, const T* __restrict__ P5) {
+  using V = typename Vec16<T>::type;
+  constexpr int VW = Vec16<T>::n;
+  const int DV = D / VW;
   const int64_t gid = (int64_t)bx_ * blockDim.x + threadIdx.x;
-  if (gid >= Bc * N * D) return;
-  const int a = (int)(gid % D);
-  const int64_t bi = gid / D;
+  if (gid >= Bc * N * DV) return;
+  const int a = (int)(gid % DV) * VW;
+  const int64_t bi = gid / DV;
   const int i = (int)(bi % N);
   const T* p = P + bi * C * D + a;
+  const T* p5 = P5 ? P5 + bi * 5 * D + a : nullptr;
   const T* fi = Fin + bi * C * D + a;
   T* f = Fout + bi * C * D + a;
-  const T t = tanh_t(p[0]);
-  const T dt = T(1) - t * t;
-  f[0] = (from_spin ? E_spin[(i < n_up ? 0 : 1) * D + a] : fi[0]) + t;
-  if (C > 1) {
-    T ss = 0;
-    for (int c = 1; c < C - 1; ++c) {
-      const T pc = p[(int64_t)c * D];
-      ss += pc * pc;
-      f[(int64_t)c * D] = (from_spin ? T(0) : fi[(int64_t)c * D]) + dt * pc;
+  __nv_bfloat16* fb = Fbf ? Fbf + bi * C * D + a : nullptr;
+  auto load = [](const T* q, T (&v)[VW]) {
+    const V x = *reinterpret_cast<const V*>(q);
+#pragma unroll
+    for (int k = 0; k < VW; ++k) v[k] = reinterpret_cast<const T*>(&x)[k];
+  };
+  auto load_p = [&](int c, T (&v)[VW]) {
+    const int x = c - 3 * i;  // 1, 2, 3: the electron's own coordinates
+    const int slot = c == 0 ? 0 : c == C - 1 ? 4 : x >= 1 && x <= 3 ? x : -1;
+    load(p5 && slot >= 0 ? p5 + (int64_t)slot * D : p + (int64_t)c * D, v);
+  };
+  auto store = [&](int c, const T (&v)[VW]) {
+    V x;
+#pragma unroll
+    for (int k = 0; k < VW; ++k) reinterpret_cast<T*>(&x)[k] = v[k];
+    *reinterpret_cast<V*>(f + (int64_t)c * D) = x;
+    if (fb) {  // BF16 copy of the embeddings: the input of the next node-map GEMM
+      __align__(8) __nv_bfloat16 h[VW];
+#pragma unroll
+      for (int k = 0; k < VW; ++k) h[k] = __float2bfloat16_rn((float)v[k]);
+      if constexpr (VW == 4)
+        *reinterpret_cast<uint2*>(fb + (int64_t)c * D) = *reinterpret_cast<const uint2*>(h);
+      else
+#pragma unroll
+        for (int k = 0; k < VW; ++k) fb[(int64_t)c * D + k] = h[k];
     }
-    const int64_t cl = (int64_t)(C - 1) * D;
-    f[cl] = (from_spin ? T(0) : fi[cl]) + dt * p[cl] - T(2) * t * dt * ss;
+  };
+  T t[VW], dt[VW], ss[VW], pv[VW], fv[VW];
+  load_p(0, pv);
+  if (from_spin) {
+#pragma unroll
+    for (int k = 0; k < VW; ++k) fv[k] = E_spin[(i < n_up ? 0 : 1) * D + a + k];
+  } else {
+    load(fi, fv);
   }
-  if (Fbf) {  // BF16 copy of the embeddings: the input of the next node-map GEMM
-    __nv_bfloat16* fb = Fbf + bi * C * D + a;
-    for (int c = 0; c < C; ++c) fb[(int64_t)c * D] = __float2bfloat16_rn((float)f[(int64_t)c * D]);
+#pragma unroll
+  for (int k = 0; k < VW; ++k) {
+    t[k] = tanh_t(pv[k]);
+    dt[k] = T(1) - t[k] * t[k];
+    ss[k] = 0;
+    fv[k] = fv[k] + t[k];
   }
+  store(0, fv);
+  if (C == 1) return;
+  for (int c0 = 1; c0 < C - 1; c0 += kUpdBatch) {
+    T pb[kUpdBatch][VW], fq[kUpdBatch][VW];
+#pragma unroll
+    for (int u = 0; u < kUpdBatch; ++u) {
+      const int c = min(c0 + u, C - 2);
+      load_p(c, pb[u]);
+      if (from_spin) {
+#pragma unroll
+        for (int k = 0; k < VW; ++k) fq[u][k] = T(0);
+      } else {
+        load(fi + (int64_t)c * D, fq[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kUpdBatch; ++u) {
+      if (c0 + u >= C - 1) break;
+#pragma unroll
+      for (int k = 0; k < VW; ++k) {
+        ss[k] += pb[u][k] * pb[u][k];
+        fq[u][k] = fq[u][k] + dt[k] * pb[u][k];
+      }
+      store(c0 + u, fq[u]);
+    }
+  }
+  load_p(C - 1, pv);
+  if (from_spin) {
+#pragma unroll
+    for (int k = 0; k < VW; ++k) fv[k] = T(0);
+  } else {
+    load(fi + (int64_t)(C - 1) * D, fv);
+  }
+#pragma unroll
+  for (int k = 0; k < VW; ++k) fv[k] = fv[k] + dt[k] * pv[k] - T(2) * t[k] * dt[k] * ss[k];
+  store(C - 1, fv);
 }
 
 template <class T>
 __global__ void update_kernel(const T* __restrict__ P, const T* Fin, T* Fout, const T* __restrict__ E_spin,
                               int64_t Bc, int N, int n_up, int C, int D, int from_spin,
                               __nv_bfloat16* __restrict__ Fbf) {
-  update_kernel_body<T>(blockIdx.x, blockIdx.y, gridDim.x, P, Fin, Fout, E_spin, Bc, N, n_up, C, D, from_spin, Fbf);
+  update_kernel_body<T>(blockIdx.x, blockIdx.y, gridDim.x, P, Fin, Fout, E_spin, Bc, N, n_up, C, D, from_spin, Fbf,
+                        nullptr);
 }
 
 // One launch over several molecules: block b runs entry m of the table.
@@ -1068,7 +1151,7 @@ __global__ void update_kernel_group(const __grid_constant__ Grp<update_kernel_ar
   int64_t l_;
   const int m_ = grp_find(g, blockIdx.x, l_);
   GRP_STATIC(m_, const auto& a_ = g.a[K_];
-             update_kernel_body<T>(grp_bx(g, K_, l_), grp_by(g, K_, l_), g.nbx[K_], a_.P, a_.Fin, a_.Fout, a_.E_spin, a_.Bc, a_.N, a_.n_up, a_.C, a_.D, a_.from_spin, a_.Fbf);)
+             update_kernel_body<T>(grp_bx(g, K_, l_), grp_by(g, K_, l_), g.nbx[K_], a_.P, a_.Fin, a_.Fout, a_.E_spin, a_.Bc, a_.N, a_.n_up, a_.C, a_.D, a_.from_spin, a_.Fbf, a_.P5);)
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int64_t n) {
@@ -2387,7 +2470,7 @@ cudaError_t launch_update(const dq_handle_s& h, const FwdDims& d, const T* param
 template <class T>
 cudaError_t launch_update_io(const dq_handle_s& h, const FwdDims& d, const T* params, bool from_spin, const T* P,
                              const T* Fin, T* Fout, cudaStream_t s, void* Fbf) {
-  update_kernel<T><<<blocks(d.Bc * d.N * d.D, 256), 256, 0, s>>>(P, Fin, Fout, params + std::max<int64_t>(h.off.E_spin, 0), d.Bc, d.N,
+  update_kernel<T><<<blocks(d.Bc * d.N * (d.D / Vec16<T>::n), 256), 256, 0, s>>>(P, Fin, Fout, params + std::max<int64_t>(h.off.E_spin, 0), d.Bc, d.N,
                                                                  d.n_up, d.C, d.D, from_spin ? 1 : 0,
                                                                  static_cast<__nv_bfloat16*>(Fbf));
   return cudaGetLastError();
@@ -2655,7 +2738,7 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
                                               reinterpret_cast<const float*>(m[k].b.Z),
                                               reinterpret_cast<const float*>(m[k].b.ew),
                                               reinterpret_cast<const float*>(m[k].b.geo), out_of(m[k]),
-                                              sizeof(TO) == 2, s);
+                                              m[k].b.msg5, sizeof(TO) == 2, s);
         if (e != cudaSuccess) return e;
         continue;
       }
@@ -2684,7 +2767,7 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
     smem = std::max(smem, lay.total_bytes);
     ent[ne++] = Ent{{m[k].b.Z, m[k].b.z0, m[k].b.ew, m[k].b.geo, m[k].params + h.off.layer[l].Y, h.d_pair_of, d.N,
                      d.n_up, d.M, d.C, d.D, h.edges.n_all, h.edges.n_ee, z_const && !h.el_init ? 1 : 0, stage_w1 ? 1 : 0,
-                     out_of(m[k])},
+                     out_of(m[k]), static_cast<TO*>(m[k].b.msg5)},
                     d.Bc, d.D / L, L, lay.total_bytes, 0};
   }
   if (ne == 0) return cudaSuccess;
@@ -2742,8 +2825,9 @@ cudaError_t launch_update_group(const MolFwd<T>* m, int n, bool from_spin, cudaS
     const FwdDims& d = m[k].d;
     if (d.Bc <= 0) continue;
     g.add({m[k].b.Z, m[k].b.F, m[k].b.F, m[k].params + std::max<int64_t>(m[k].h->off.E_spin, 0), d.Bc, d.N, d.n_up, d.C, d.D,
-           from_spin && !m[k].h->el_init ? 1 : 0, static_cast<__nv_bfloat16*>(m[k].b.F_bf)},
-          blocks(d.Bc * d.N * d.D, 256));
+           from_spin && !m[k].h->el_init ? 1 : 0, static_cast<__nv_bfloat16*>(m[k].b.F_bf),
+           m[k].b.un5},
+          blocks(d.Bc * d.N * (d.D / Vec16<T>::n), 256));
   }
   if (g.n == 0) return cudaSuccess;
   cudaError_t e = check_group(g);

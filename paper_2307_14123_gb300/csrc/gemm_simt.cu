@@ -37,7 +37,8 @@ __device__ __forceinline__ int64_t row_offset(const RowMap& m, int64_t r) {
 template <class T, int BM, int BN, int BK, bool XA, bool WA>
 __global__ void __launch_bounds__(256)
     gemm_nt_kernel(const T* __restrict__ X, RowMap mx, const T* __restrict__ W, const T* __restrict__ bias,
-                   int bias_period, T* __restrict__ Y, RowMap my, int64_t rows, int n_out, int K, int accumulate) {
+                   int bias_period, T* __restrict__ Y, RowMap my, int64_t rows, int n_out, int K, int ldw,
+                   int accumulate) {
   using V = typename Vec<T>::type;
   constexpr int VEC = Vec<T>::n;
   constexpr int NT = 256;
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(256)
     b_kv[i] = l % KV;
     const int n = col0 + b_row[i];
     b_ok[i] = n < n_out;
-    b_ptr[i] = W + (b_ok[i] ? (int64_t)n * K : 0) + b_kv[i] * VEC;
+    b_ptr[i] = W + (b_ok[i] ? (int64_t)n * ldw : 0) + b_kv[i] * VEC;
   }
 
   V ra[LA], rb[LB];
@@ -190,7 +191,7 @@ template <int BM, int BN>
 __global__ void __launch_bounds__(256)
     gemm_nt_f64_kernel(const double* __restrict__ X, RowMap mx, const double* __restrict__ W,
                        const double* __restrict__ bias, int bias_period, double* __restrict__ Y, RowMap my, int64_t rows,
-                       int n_out, int K, int accumulate) {
+                       int n_out, int K, int ldw, int accumulate) {
   constexpr int NT = 256;
   constexpr int CT = BN < 16 ? BN : 16;  // threads along the columns
   constexpr int TM = BM * CT / NT, TN = BN / CT;
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int i = 0; i < LB; ++i) {
     const int n = col0 + lr0 + i * (NT / F64_BK);
-    b_ptr[i] = n < n_out ? W + (int64_t)n * K + kk0 : nullptr;
+    b_ptr[i] = n < n_out ? W + (int64_t)n * ldw + kk0 : nullptr;
   }
   double ra[LA], rb[LB];
   auto load = [&](int k0) {
@@ -271,12 +272,13 @@ namespace {
 // The FP64 tile: the one that gives the busiest SM the fewest multiply-adds (its share of the
 // tiles, rounded up, times the tile's area, padding included); the larger tile where two agree.
 cudaError_t gemm_f64_dispatch(const double* X, RowMap mx, const double* W, const double* bias, int bias_period,
-                              double* Y, RowMap my, int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s) {
+                              double* Y, RowMap my, int64_t rows, int n_out, int K, int ldw, bool accumulate,
+                              cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   using Kern = void (*)(const double*, RowMap, const double*, const double*, int, double*, RowMap, int64_t, int, int,
-                        int);
+                        int, int);
   struct Tile {
     int bm, bn;
     Kern kern;
@@ -295,45 +297,46 @@ cudaError_t gemm_f64_dispatch(const double* X, RowMap mx, const double* W, const
     }
   }
   const dim3 grid((unsigned)((rows + best->bm - 1) / best->bm), (unsigned)((n_out + best->bn - 1) / best->bn));
-  best->kern<<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate ? 1 : 0);
+  best->kern<<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, accumulate ? 1 : 0);
   return cudaGetLastError();
 }
 
 template <class T, int BM, int BN, int BK>
 cudaError_t gemm_dispatch(const T* X, RowMap mx, const T* W, const T* bias, int bias_period, T* Y, RowMap my,
-                          int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s) {
+                          int64_t rows, int n_out, int K, int ldw, bool accumulate, cudaStream_t s) {
   constexpr int VEC = Vec<T>::n;
   const bool xa = (uintptr_t)X % 16 == 0 && mx.ld % VEC == 0 && mx.seg_stride % VEC == 0;
-  const bool wa = (uintptr_t)W % 16 == 0;
+  const bool wa = (uintptr_t)W % 16 == 0 && ldw % VEC == 0;
   dim3 grid((unsigned)((rows + BM - 1) / BM), (unsigned)((n_out + BN - 1) / BN));
   const int acc = accumulate ? 1 : 0;
   if (xa && wa)
-    gemm_nt_kernel<T, BM, BN, BK, true, true><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, acc);
+    gemm_nt_kernel<T, BM, BN, BK, true, true><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, acc);
   else if (xa)
-    gemm_nt_kernel<T, BM, BN, BK, true, false><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, acc);
+    gemm_nt_kernel<T, BM, BN, BK, true, false><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, acc);
   else if (wa)
-    gemm_nt_kernel<T, BM, BN, BK, false, true><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, acc);
+    gemm_nt_kernel<T, BM, BN, BK, false, true><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, acc);
   else
-    gemm_nt_kernel<T, BM, BN, BK, false, false><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, acc);
+    gemm_nt_kernel<T, BM, BN, BK, false, false><<<grid, 256, 0, s>>>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, acc);
   return cudaGetLastError();
 }
 }  // namespace
 
 template <class T>
 cudaError_t gemm_nt(const T* X, RowMap mx, const T* W, const T* bias, int bias_period, T* Y, RowMap my,
-                    int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s) {
+                    int64_t rows, int n_out, int K, bool accumulate, cudaStream_t s, int ldw) {
+  if (ldw == 0) ldw = K;
   if (rows <= 0 || n_out <= 0) return cudaSuccess;
   if (K % 8 != 0 || bias_period <= 0) return cudaErrorInvalidValue;
   if constexpr (sizeof(T) == 4) {
-    return gemm_dispatch<T, 128, 128, 8>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate, s);
+    return gemm_dispatch<T, 128, 128, 8>(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, accumulate, s);
   } else {
-    return gemm_f64_dispatch(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, accumulate, s);
+    return gemm_f64_dispatch(X, mx, W, bias, bias_period, Y, my, rows, n_out, K, ldw, accumulate, s);
   }
 }
 
 template cudaError_t gemm_nt<float>(const float*, RowMap, const float*, const float*, int, float*, RowMap,
-                                    int64_t, int, int, bool, cudaStream_t);
+                                    int64_t, int, int, bool, cudaStream_t, int);
 template cudaError_t gemm_nt<double>(const double*, RowMap, const double*, const double*, int, double*,
-                                     RowMap, int64_t, int, int, bool, cudaStream_t);
+                                     RowMap, int64_t, int, int, bool, cudaStream_t, int);
 
 }  // namespace dq

@@ -855,12 +855,12 @@ constexpr size_t tc_smem_bytes() { return 1024 + TC_STAGES * (TC_TILE_A + TC_TIL
 }  // namespace
 
 cudaError_t gemm_bf16_tc(const void* X, int64_t rows, int K, int64_t ldx, const void* W, int n_out, const float* bias,
-                         int bias_period, float* Y, int64_t ldy, unsigned int* status, cudaStream_t s) {
+                         int bias_period, float* Y, int64_t ldy, unsigned int* status, cudaStream_t s, int64_t ldw) {
   if (rows <= 0 || n_out <= 0) return cudaSuccess;
-  if (K % TC_BK || ldx % 8 || (uintptr_t)X % 16 || (uintptr_t)W % 16 || bias_period <= 0)
+  if (K % TC_BK || ldx % 8 || ldw % 8 || (uintptr_t)X % 16 || (uintptr_t)W % 16 || bias_period <= 0)
     return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, X, rows, K, ldx, TC_BM) || !make_map(&mb, W, n_out, K, K, TC_BN)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, X, rows, K, ldx, TC_BM) || !make_map(&mb, W, n_out, K, ldw ? ldw : K, TC_BN)) return cudaErrorInvalidValue;
   const size_t smem = tc_smem_bytes();
   cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -11,7 +11,7 @@
 // One CTA per (walker, 32 features), a lane per feature, 16 warps.  The senders are taken one
 // spin block at a time: pass p holds the senders of block p, which give a receiver of block p its
 // same-spin message and every other receiver its opposite-spin one.  Per pass, w_ij, w'_ij and
-// w''_ij of the block's senders and all receivers are copied into shared memory as [j][i][32]
+// w''_ij of the block's senders and all receivers are copied into shared memory as [i][j][32]
 // (16-byte asynchronous copies; rows past the block and the diagonal are zero).  A warp task
 // owns the 3 EPT coordinate channels of EPT consecutive electrons (one more task the value and
 // Laplacian channels): it loads z_j[c] of the block's NBS sender slots for them into registers
@@ -25,7 +25,10 @@
 // The general kernel (forward.cu) streams the senders' node channels four senders at a time
 // through 4-byte copies per lane, with the w tables of all N^2 pairs resident; here z lives in
 // registers, read once, and only one spin block's tables are resident (at 28 electrons this
-// kernel takes half the general kernel's time).
+// kernel takes half the general kernel's time).  In the receiver loop every w sits at a
+// compile-time offset ([i][sender slot][32]), a pair's geometry is one 16-byte load and an output a
+// 32-bit offset from the walker's base: with run-time strides and a pointer per store the
+// addresses took more instructions than the sums (all messages of 333 C4H4 walkers 8.5 -> 7.5 ms).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -45,21 +48,22 @@ struct MLArgs {
   const float* geo;    // [Bc][E][4] distance and unit vector of every edge
   const float* Y;      // [M][D] nucleus embeddings of the layer
   const int* pair_of;  // [N][N] edge of (i, j), -1 on the diagonal
-  void* msg;           // [Bc][N][C][3D] messages [same spin | opposite spin | nuclei]
+  void* msg;           // [Bc][N][C][3D] messages [same spin | opposite spin | nuclei], or with msg5
+                       // [Bc][N][C][2D] without the nuclei's
+  void* msg5;          // [Bc][N][5][3D] the value, own-coordinate and Laplacian rows (nullptr: in msg)
   int N, n_up, M, C, D, E, n_ee;
   int stage_w1;        // w' and w'' tables in shared memory (else read from global memory)
 };
 
 // Shared-memory layout in floats (the pair table in ints at the same scale).
 struct MLSmem {
-  int ps, us, id, z0c, zsf, spb, spc, lap, w0, w1, w2, total_bytes;
+  int ps, ug, z0c, zsf, spb, spc, lap, w0, w1, w2, total_bytes;
 };
 __host__ __device__ inline MLSmem ml_layout(int N, int NBS, bool stage_w1) {
   MLSmem m{};
   int o = 0;
+  m.ug = o; o += N * N * 4;
   m.ps = o; o += N * N;
-  m.us = o; o += N * N * 3;
-  m.id = o; o += N * N;
   m.z0c = o; o += N * kMLLanes;
   m.zsf = o; o += 3 * N * kMLLanes;
   m.spb = o; o += 3 * N * kMLLanes;
@@ -91,16 +95,15 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
   const int N = a.N, C = a.C, D = a.D, M = a.M, n_up = a.n_up, n_ee = a.n_ee;
   const MLSmem lay = ml_layout(N, NBS, SW1);
   int* Ps = reinterpret_cast<int*>(ml_smem + lay.ps);  // [i][j] edge
-  float* Us = ml_smem + lay.us;                        // [i][j][3] u_ij (zero diagonal)
-  float* Id = ml_smem + lay.id;                        // [i][j] 1 / d_ij
+  float4* Ug = reinterpret_cast<float4*>(ml_smem + lay.ug);  // [i][j] u_ij and 1 / d_ij (zero diagonal)
   float* Z0c = ml_smem + lay.z0c;                      // [j][32] z_j[0]
   float* Zsf = ml_smem + lay.zsf;                      // [j][x][32] dz_j / dr_j,x
   float* SPb = ml_smem + lay.spb;                      // [i][x][32] (b) of the pass
   float* SPc = ml_smem + lay.spc;                      // [i][32] (c) of the pass
   float* LAP = ml_smem + lay.lap;                      // [i][32] Laplacian-channel contraction
-  float* W0 = ml_smem + lay.w0;                        // [jj][i][32] w of the pass's senders
-  float* W1 = ml_smem + lay.w1;                        // [jj][i][32] w'
-  float* W2 = ml_smem + lay.w2;                        // [jj][i][32] w''
+  float* W0 = ml_smem + lay.w0;                        // [i][jj][32] w of the pass's NBS sender slots
+  float* W1 = ml_smem + lay.w1;                        // [i][jj][32] w'
+  float* W2 = ml_smem + lay.w2;                        // [i][jj][32] w''
   constexpr bool stage_w1 = SW1;
 
   const int64_t b = blockIdx.x;
@@ -110,7 +113,15 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
   const float* Zb = a.Z + b * (int64_t)N * C * D + f0 + lane;
   const float* Yd = a.Y + f0 + lane;
   const float* Gb = a.geo + b * (int64_t)a.E * 4;
-  TO* mb = static_cast<TO*>(a.msg) + b * (int64_t)N * C * 3 * D + f0 + lane;
+  const int64_t mp = (a.msg5 ? 2 : 3) * (int64_t)D;  // row pitch of msg
+  const uint32_t mp32 = (uint32_t)mp;                // (a walker's N C rows: below 2^32 elements)
+  TO* mbw = static_cast<TO*>(a.msg) + b * (int64_t)N * C * mp + f0;  // lane-independent
+  TO* mb = static_cast<TO*>(a.msg) + b * (int64_t)N * C * mp + f0 + lane;
+  TO* m5 = a.msg5 ? static_cast<TO*>(a.msg5) + b * (int64_t)N * 15 * D + f0 + lane : nullptr;
+  // the row of receiver i's channel c, slot its place among the five rows apart
+  auto special = [&](int i, int c, int slot) {
+    return m5 ? m5 + ((int64_t)i * 5 + slot) * 3 * D : mb + ((int64_t)i * C + c) * mp;
+  };
   const int NN = N * N;
 
   // this CTA's slices of the node channels and filters into L2
@@ -133,10 +144,7 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       u2 = sg * g.w;
       id = 1.f / g.x;
     }
-    Us[k * 3] = u0;
-    Us[k * 3 + 1] = u1;
-    Us[k * 3 + 2] = u2;
-    Id[k] = id;
+    Ug[k] = make_float4(u0, u1, u2, id);
   }
   for (int j = warp; j < N; j += NW) {
     const float* zj = Zb + (int64_t)j * C * D;
@@ -173,11 +181,15 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
         sl = fmaf(w2v[u] + 2.f * w1v[u] / g[0], yv[u], sl);
       }
     }
-    TO* o = mb + (int64_t)i * C * 3 * D + 2 * D;
-    for (int c = 0; c < C; ++c) {
-      const float v = c == 0 ? sv : c == C - 1 ? sl : c == 1 + 3 * i ? sx : c == 2 + 3 * i ? sy : c == 3 + 3 * i ? sz : 0.f;
-      store_out(o + (int64_t)c * 3 * D, v * nuM);
+    if (m5 == nullptr) {
+      TO* o = mb + (int64_t)i * C * mp + 2 * D;
+      for (int c = 0; c < C; ++c) store_out(o + (int64_t)c * mp, 0.f);
     }
+    store_out(special(i, 0, 0) + 2 * D, sv * nuM);
+    store_out(special(i, 1 + 3 * i, 1) + 2 * D, sx * nuM);
+    store_out(special(i, 2 + 3 * i, 2) + 2 * D, sy * nuM);
+    store_out(special(i, 3 + 3 * i, 3) + 2 * D, sz * nuM);
+    store_out(special(i, C - 1, 4) + 2 * D, sl * nuM);
   }
   __syncthreads();  // pair table, unit vectors, z_j[0]
 
@@ -186,7 +198,7 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
   const float* ew_row = a.ew + b * (int64_t)a.E * 3 * D + f0;  // lane-independent row base
   for (int pass = 0; pass < 2; ++pass) {
     const int j0 = pass == 0 ? 0 : n_up, jn = pass == 0 ? n_up : N - n_up;
-    // ---- the pass's filter tables: row (jj, i) holds w_{i, j0 + jj} for the 32 features, as
+    // ---- the pass's filter tables: row (i, jj) holds w_{i, j0 + jj} for the 32 features, as
     // eight 16-byte copies (lane / 8 picks one of four rows, lane % 8 the chunk) ----
     {
       const int rows = NBS * N;
@@ -194,7 +206,7 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       for (int r0 = warp * 4; r0 < rows; r0 += NW * 4) {
         const int r = r0 + sub;
         if (r < rows) {
-          const int jj = r / N, i = r - (r / N) * N;
+          const int i = r / NBS, jj = r % NBS;
           const int j = j0 + jj;
           const int p = (jj < jn && i != j) ? Ps[i * N + j] : -1;
           const float* src = ew_row + (int64_t)(p >= 0 ? p : 0) * 3 * D + ch;
@@ -210,7 +222,7 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
     }
     __syncthreads();
     auto w1_at = [&](int i, int jj) -> float {  // w'_{i, j0 + jj} of this lane's feature
-      if (stage_w1) return W1[(jj * N + i) * 32 + lane];
+      if (stage_w1) return W1[(i * NBS + jj) * 32 + lane];
       const int j = j0 + jj;
       return i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
     };
@@ -247,30 +259,45 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
           const int e = e0 + s;
           if (e >= N) break;
           float b0 = 0.f, b1 = 0.f, b2 = 0.f, sv = 0.f;
-          float w2v[SW1 ? 1 : NBS];  // w'' from global memory when the tables are not staged
-          if (!SW1) {
+          // w' and w'' of eight senders at a time: from global memory (when the tables are not
+          // staged) their loads are issued together
+          constexpr int CH = SW1 ? NBS : 8;
 #pragma unroll
-            for (int jj = 0; jj < NBS; ++jj) {
-              const int j = j0 + jj;
-              w2v[SW1 ? 0 : jj] = (jj < jn && j != e) ? EWb[((int64_t)Ps[e * N + j] * 3 + 2) * D] : 0.f;
+          for (int jc = 0; jc < NBS; jc += CH) {
+            float w1v[CH], w2v[CH];
+#pragma unroll
+            for (int u = 0; u < CH; ++u) {
+              const int jj = jc + u, j = j0 + jj;
+              if (SW1) {
+                w1v[u] = W1[(e * NBS + jj) * 32 + lane];
+                w2v[u] = W2[(e * NBS + jj) * 32 + lane];
+              } else {
+                const float* w = EWb + ((int64_t)(jj < jn && j != e ? Ps[e * N + j] : 0) * 3 + 1) * D;
+                w1v[u] = jj < jn && j != e ? w[0] : 0.f;
+                w2v[u] = jj < jn && j != e ? w[D] : 0.f;
+              }
             }
-          }
 #pragma unroll
-          for (int jj = 0; jj < NBS; ++jj) {
-            if (jj >= jn) break;
-            const int j = j0 + jj;
-            const float v1 = w1_at(e, jj);
-            const float* uu = Us + (e * N + j) * 3;
-            const float z0 = Z0c[j * 32 + lane];
-            b0 = fmaf(v1 * uu[0], z0, b0);
-            b1 = fmaf(v1 * uu[1], z0, b1);
-            b2 = fmaf(v1 * uu[2], z0, b2);
-            if (j == e) continue;
-            const float* zs = Zsf + (j * 3) * 32 + lane;
-            const float cr = uu[0] * (zr[3 * s][jj] - zs[0]) + uu[1] * (zr[3 * s + 1][jj] - zs[32]) +
-                             uu[2] * (zr[3 * s + 2][jj] - zs[64]);
-            const float w2 = SW1 ? W2[(jj * N + e) * 32 + lane] : w2v[SW1 ? 0 : jj];
-            sv += (2.f * w2 + 4.f * v1 * Id[e * N + j]) * z0 + 2.f * v1 * cr;
+            for (int u = 0; u < CH; ++u) {
+              const int jj = jc + u;
+              if (jj >= NBS || jj >= jn) break;
+              const int j = j0 + jj;
+              const float v1 = w1v[u];
+              const float4 uu = Ug[e * N + j];
+              const float z0 = Z0c[j * 32 + lane];
+              b0 = fmaf(v1 * uu.x, z0, b0);
+              b1 = fmaf(v1 * uu.y, z0, b1);
+              b2 = fmaf(v1 * uu.z, z0, b2);
+              if (j == e) continue;
+              const float* zs = Zsf + (j * 3) * 32 + lane;
+              // (every operation's rounding is fixed: the sums become BF16 operands, which a last bit
+              // can move)
+              const float cr = __fmaf_rn(uu.z, zr[3 * s + 2][jj] - zs[64],
+                                         __fmaf_rn(uu.x, zr[3 * s][jj] - zs[0], __fmul_rn(uu.y, zr[3 * s + 1][jj] - zs[32])));
+              const float q = SW1 ? __fmaf_rn(2.f, w2v[u], __fmul_rn(4.f * v1, uu.w))
+                                  : __fmaf_rn(4.f * v1, uu.w, 2.f * w2v[u]);
+              sv = __fadd_rn(sv, __fmaf_rn(2.f * v1, cr, __fmul_rn(q, z0)));
+            }
           }
           SPb[(e * 3) * 32 + lane] = b0;
           SPb[(e * 3 + 1) * 32 + lane] = b1;
@@ -278,37 +305,49 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
           SPc[e * 32 + lane] = sv;
         }
         __syncwarp();
-        for (int i = 0; i < N; ++i) {
+        // the receivers: w rows at compile-time offsets, outputs at 32-bit offsets of the walker's base
+        const float* wr = W0 + lane;
+        const float4* ug = Ug + e0;
+        uint32_t off = (uint32_t)c0 * mp32 + lane;
+        float w1n[EPT];  // w'_{i, e0 + s} of the next receiver
+#pragma unroll
+        for (int s = 0; s < EPT; ++s) w1n[s] = SW1 ? 0.f : w1_at(0, ja[s]);
+#pragma unroll 1
+        for (int i = 0; i < N; ++i, wr += NBS * 32, ug += N, off += (uint32_t)C * mp32) {
           float acc[CB];
 #pragma unroll
           for (int q = 0; q < CB; ++q) acc[q] = 0.f;
-          const float* wr = W0 + i * 32 + lane;
 #pragma unroll
           for (int jj = 0; jj < NBS; ++jj) {
-            const float w = wr[jj * N * 32];
+            const float w = wr[jj * 32];
 #pragma unroll
             for (int q = 0; q < CB; ++q) acc[q] = fmaf(w, zr[q][jj], acc[q]);
           }
+          const bool same = (i < n_up) == (pass == 0);
+          const float nu = same ? nu_same : nu_opp;
+          const uint32_t slot = same ? 0u : (uint32_t)D;
 #pragma unroll
           for (int s = 0; s < EPT; ++s) {
             const int e = e0 + s;
             if (e >= N) break;
             // (a): -w'_ie z_e[0] u_ie,x (w'_ii = 0: nothing on the receiver's own channels)
-            const float pa = (SW1 ? W1[(ja[s] * N + i) * 32 + lane] : w1_at(i, ja[s])) * za[s];
-            const float* ue = Us + (i * N + e) * 3;
+            const float w1 = SW1 ? W1[(i * NBS + ja[s]) * 32 + lane] : w1n[s];
+            if (!SW1 && i + 1 < N) w1n[s] = w1_at(i + 1, ja[s]);
+            const float pa = w1 * za[s];
+            const float4 ue = ug[s];
+            acc[3 * s] = fmaf(-pa, ue.x, acc[3 * s]);
+            acc[3 * s + 1] = fmaf(-pa, ue.y, acc[3 * s + 1]);
+            acc[3 * s + 2] = fmaf(-pa, ue.z, acc[3 * s + 2]);
+            if (e == i) {  // (b): the receiver's own coordinates, rows apart when the messages are split
+              TO* o = special(i, 1 + 3 * i, 1) + slot;
+              const int64_t pitch = m5 ? 3 * (int64_t)D : mp;
 #pragma unroll
-            for (int x = 0; x < 3; ++x) acc[3 * s + x] = fmaf(-pa, ue[x], acc[3 * s + x]);
-            if (e == i) {  // (b): the receiver's own coordinates
+              for (int x = 0; x < 3; ++x) store_out(o + x * pitch, (acc[3 * s + x] + SPb[(i * 3 + x) * 32 + lane]) * nu);
+            } else {
 #pragma unroll
-              for (int x = 0; x < 3; ++x) acc[3 * s + x] += SPb[(i * 3 + x) * 32 + lane];
+              for (int x = 0; x < 3; ++x) store_out(mbw + (off + slot + (3 * s + x) * mp32), acc[3 * s + x] * nu);
             }
           }
-          const bool same = (i < n_up) == (pass == 0);
-          const float nu = same ? nu_same : nu_opp;
-          TO* o = mb + ((int64_t)i * C + c0) * 3 * D + (same ? 0 : D);
-#pragma unroll
-          for (int q = 0; q < CB; ++q)
-            if (e0 + q / 3 < N) store_out(o + (int64_t)q * 3 * D, acc[q] * nu);
         }
       } else {
         // the value channel (z_j[0] from shared memory) and the Laplacian channel, with (c)
@@ -320,16 +359,16 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
         }
         for (int i = 0; i < N; ++i) {
           float av = 0.f, al = 0.f;
-          const float* wr = W0 + i * 32 + lane;
+          const float* wr = W0 + i * NBS * 32 + lane;
 #pragma unroll
           for (int jj = 0; jj < NBS; ++jj) {
-            const float w = wr[jj * N * 32];
+            const float w = wr[jj * 32];
             av = fmaf(w, zv[jj], av);
             al = fmaf(w, zl[jj], al);
           }
           const bool same = (i < n_up) == (pass == 0);
           const float nu = same ? nu_same : nu_opp;
-          store_out(mb + (int64_t)i * C * 3 * D + (same ? 0 : D), av * nu);
+          store_out(special(i, 0, 0) + (same ? 0 : D), av * nu);
           LAP[i * 32 + lane] = al;  // completed with (c) after every task has written SPc
         }
       }
@@ -340,7 +379,7 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       const bool same = (i < n_up) == (pass == 0);
       const float nu = same ? nu_same : nu_opp;
       const float al = LAP[i * 32 + lane] + SPc[i * 32 + lane];
-      store_out(mb + ((int64_t)i * C + C - 1) * 3 * D + (same ? 0 : D), al * nu);
+      store_out(special(i, C - 1, 4) + (same ? 0 : D), al * nu);
     }
     __syncthreads();  // the tables are rewritten by the next pass
   }
@@ -369,13 +408,13 @@ bool messages_large_supported(const dq_handle_s& h, const FwdDims& d) {
 }
 
 cudaError_t launch_messages_large(const dq_handle_s& h, const FwdDims& d, const float* params, int l,
-                                  const float* Z, const float* ew, const float* geo, void* msg, bool bf16_out,
-                                  cudaStream_t s) {
+                                  const float* Z, const float* ew, const float* geo, void* msg, void* msg5,
+                                  bool bf16_out, cudaStream_t s) {
   if (d.Bc <= 0) return cudaSuccess;
   if (!messages_large_supported(h, d)) return cudaErrorInvalidValue;
   const int nb = std::max(d.n_up, d.N - d.n_up);
   const int nbs = ml_nbs(nb);
-  MLArgs a{Z, ew, geo, params + h.off.layer[l].Y, h.d_pair_of, msg, d.N, d.n_up, d.M, d.C, d.D,
+  MLArgs a{Z, ew, geo, params + h.off.layer[l].Y, h.d_pair_of, msg, msg5, d.N, d.n_up, d.M, d.C, d.D,
            h.edges.n_all, h.edges.n_ee, 1};
   if (ml_layout(d.N, nbs, true).total_bytes > 220 * 1024) a.stage_w1 = 0;
   // register tiles of sender slots x 3 EPT channels (72 to 84 values) in 16 warps of 128 registers
