@@ -393,6 +393,11 @@ bool messages_large_supported(const dq_handle_s& h, const FwdDims& d);
 cudaError_t launch_messages_large(const dq_handle_s& h, const FwdDims& d, const float* params, int l,
                                   const float* Z, const float* ew, const float* geo, void* msg, void* msg5,
                                   bool bf16_out, cudaStream_t s);
+// Jet messages of constant node channels z0 [2][D] (layer 0 on spin embeddings, FP32 modes;
+// messages_const.cu); msg, msg5 as above.
+cudaError_t launch_messages_const(const dq_handle_s& h, const FwdDims& d, const float* params, int l, const float* z0,
+                                  const float* ew, const float* geo, void* msg, void* msg5, bool bf16_out,
+                                  cudaStream_t s);
 cudaError_t launch_layer_fused(const dq_handle_s& h, const FwdDims& d, const float* params, int l, bool z_const,
                                float* Z, const float* z0, const float* ew, const float* geo, float* mn,
                                const float* wg_hi, const float* wg_lo, const void* wg_bf, cudaStream_t s);

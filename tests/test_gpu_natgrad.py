@@ -178,3 +178,17 @@ def test_one_kernel_solve_over_row_splits(B):
     assert torch.equal(d, eager) and float(st[1]) <= 1e-9
     ref = oracle.natural_gradient(G, w, lam)
     assert np.linalg.norm(d.cpu().numpy() - ref) <= 2e-3 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("B", [1300, 1537])
+def test_triangular_gram_matches_oracle(B):
+    """Row counts at which half the Gram matrix saves a wave of tiles, with ragged last row and
+    column blocks; the bound of the other parity tests."""
+    wl, h = _handle("lih_fp64")
+    G, w = _synthetic(B, h.P, 41 + B)
+    lam = _damping(G, 1e-1)
+    d, st = h.natural_gradient(torch.tensor(G, dtype=torch.float32, device="cuda:0"),
+                               torch.tensor(w, dtype=torch.float32, device="cuda:0"), lam, max_iter=400, tol=1e-9)
+    ref = oracle.natural_gradient(G, w, lam)
+    assert float(st[1]) <= 1e-9
+    assert np.linalg.norm(d.cpu().numpy() - ref) <= 2e-3 * np.linalg.norm(ref)
