@@ -290,14 +290,14 @@ def peaks():
 # dram__bytes_read.sum + dram__bytes_write.sum of the jet message kernel (layer >= 1 launch) per walker,
 # from an ncu capture of the layer-1 launch on 512 N2 walkers (FP32, the tuned 4-receiver tile; summary under profiles/); None
 # once the kernel has changed since that capture.
-MSG_DRAM_BYTES_PER_WALKER = (263.570432e6 + 432.803840e6) / 512
-# the same for one launch of the fused layer kernel (layer 1 of N2, 512 walkers, the receiver-pair
-# producer design; summary under profiles/); None once the kernel has changed since that capture.
+MSG_DRAM_BYTES_PER_WALKER = None
+# the same for one launch of the fused layer kernel (layer 1 of N2, 512 walkers, tiles of whole
+# electrons; summary under profiles/); None once the kernel has changed since that capture.
 # Layer 0 (constant node channels) reads no z slabs and moves less.
-LAYER_FUSED_DRAM_BYTES_PER_WALKER = (238.052864e6 + 108.800256e6) / 512
+LAYER_FUSED_DRAM_BYTES_PER_WALKER = (234.25e6 + 108.18e6) / 512
 # the same for one launch of the sender-tiled message kernel (layer 1 of C4H4 in BF16 mode, 256
 # walkers; summary under profiles/); None once the kernel has changed since that capture.
-MSG_LARGE_DRAM_BYTES_PER_WALKER = (1.637387e9 + 0.949968e9) / 256
+MSG_LARGE_DRAM_BYTES_PER_WALKER = None
 
 
 def gemm_shapes(wl, chunk):
@@ -411,7 +411,7 @@ def roofline_for(kind, ms, n, wl, chunk, pk, how, alu, steps):
         flops = message_flops_per_walker(wl) * chunk
         peak = alu["fp32_tflops"] if wl.precision != "fp64" else alu["fp64_tflops"]
         ach = flops / t / 1e12
-        byts = (chunk * N * C * D * el * (L - 1) / L) + chunk * E * 3 * D * el + chunk * N * C * 3 * D * (2 if bf16 else el)
+        byts = (chunk * N * C * D * el * (L - 1) / L) + chunk * E * 3 * D * el + chunk * N * (2 * C + 15 if N >= 9 else 3 * C) * D * (2 if bf16 else el)
         traffic = None
         if wl.name == "n2_fp32" and MSG_DRAM_BYTES_PER_WALKER:
             traffic = MSG_DRAM_BYTES_PER_WALKER * chunk
