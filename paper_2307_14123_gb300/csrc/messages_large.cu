@@ -221,10 +221,12 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    auto w1_at = [&](int i, int jj) -> float {  // w'_{i, j0 + jj} of this lane's feature
+    // w'_{i, j0 + jj} of this lane's feature; zero past the block's senders (of an empty spin block
+    // not even slot 0 is one, and the pair table of the last receiver ends before it)
+    auto w1_at = [&](int i, int jj) -> float {
       if (stage_w1) return W1[(i * NBS + jj) * 32 + lane];
       const int j = j0 + jj;
-      return i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
+      return jj >= jn || i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
     };
     // ---- the contraction: a warp task holds the 3 EPT coordinate channels of EPT consecutive
     // electrons (channel c = 1 + 3 e + x: electron e, axis x known per register slot), and one
