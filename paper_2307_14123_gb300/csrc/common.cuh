@@ -13,6 +13,7 @@ namespace dq {
 constexpr int kMaxElec = 64;   // n_up + n_down
 constexpr int kMaxSpin = 32;   // electrons per spin channel (one warp per matrix)
 constexpr int kMaxNuc = 64;
+constexpr size_t kMaxSmem = 232448;  // shared memory of a block, static arrays included (227 KB)
 
 // Element offsets of the blocks of the flat parameter vector (layout in dqmc.h).
 struct ParamOffsets {

@@ -139,7 +139,7 @@ struct Vec16<double> {
 };
 
 // Edges per block: 32, or 16 where 32 would leave an SM fewer than four blocks (a count of blocks
-// per SM that rounds up costs less then).
+// per SM that rounds up costs less then) or would not fit (launch_edge_hidden_group).
 constexpr int kEdgesPerBlk = 32;
 constexpr int kHiddenThreads = 256;
 
@@ -2587,19 +2587,44 @@ template <class T>
 cudaError_t launch_edge_hidden_group(const MolFwd<T>* m, int n, int l, cudaStream_t s) {
   if (n > kMaxGroup) return cudaErrorInvalidValue;
   Grp<edge_hidden_kernel_args<T>> g{};
-  size_t smem = 0;
   int64_t rows_all = 0;
+  const int ej = m[0].d.C > 1 ? 3 : 1;  // all entries alike
+  auto kern = ej == 3 ? edge_hidden_kernel_group<T, 3> : edge_hidden_kernel_group<T, 1>;
   for (int k = 0; k < n; ++k) rows_all += m[k].d.Bc > 0 ? m[k].d.Bc * m[k].h->edges.n_all : 0;
+  if (rows_all == 0) return cudaSuccess;
+  auto smem_of = [&](int epb) {  // the largest entry's, with epb edges per block
+    size_t smem = 0;
+    for (int k = 0; k < n; ++k) {
+      const FwdDims& d = m[k].d;
+      if (d.Bc > 0) smem = std::max(smem, ((size_t)3 * d.Q * d.D + 3 * d.D + (size_t)2 * epb * ej * d.Q) * sizeof(T));
+    }
+    return smem;
+  };
+  // Edges per block.  Two buffers of 16 edges take the bytes of one of 32, so blocks of 16 fit every
+  // shape that a single buffer would; blocks of 32 are taken where there are rows for them, and where
+  // their buffers neither pass the shared memory of a block nor cost an SM a block (one in place of
+  // two: 1886 us against 1208 for 2048 LiH walkers in FP64 at n_rbf 32, width 96; 384 against 322
+  // for 512 N2 walkers in FP32 at n_rbf 32, width 256, jets, two layers).
+  int epb = kEdgesPerBlk;
+  if (rows_all < (int64_t)4 * kEdgesPerBlk * device_sms() || smem_of(epb) > kMaxSmem) epb /= 2;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(epb));
+  if (e != cudaSuccess) return e;
+  if (epb == kEdgesPerBlk) {
+    int occ = 0, occ_half = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kHiddenThreads, smem_of(epb));
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_half, kern, kHiddenThreads, smem_of(epb / 2));
+    if (e != cudaSuccess) return e;
+    if (occ < occ_half) epb /= 2;
+  }
+  const size_t smem = smem_of(epb);
   const int64_t grid_all = (int64_t)device_sms() * 6;  // persistent, 6 CTAs per SM, shared by row count
   for (int k = 0; k < n; ++k) {
     const dq_handle_s& h = *m[k].h;
     const FwdDims& d = m[k].d;
     if (d.Bc <= 0) continue;
-    const int ej = d.C > 1 ? 3 : 1;
     const auto& y = h.off.layer[l];
     const int64_t rows = d.Bc * h.edges.n_all;
-    const int epb = rows_all < (int64_t)4 * kEdgesPerBlk * device_sms() ? kEdgesPerBlk / 2 : kEdgesPerBlk;
-    smem = std::max(smem, ((size_t)3 * d.Q * d.D + 3 * d.D + (size_t)2 * epb * ej * d.Q) * sizeof(T));
     const int64_t nblk = (rows + epb - 1) / epb;
     int64_t share = (grid_all * rows + rows_all - 1) / rows_all;
     share = std::max<int64_t>(1, std::min(share, nblk));
@@ -2607,10 +2632,6 @@ cudaError_t launch_edge_hidden_group(const MolFwd<T>* m, int n, int l, cudaStrea
            y.W1[2], y.b1[0], y.b1[1], y.b1[2], m[k].b.eh, epb},
           share);
   }
-  if (g.n == 0) return cudaSuccess;
-  auto kern = m[0].d.C > 1 ? edge_hidden_kernel_group<T, 3> : edge_hidden_kernel_group<T, 1>;  // all entries alike
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   kern<<<(unsigned)g.blocks(), kHiddenThreads, smem, s>>>(g);
   return cudaGetLastError();
 }
