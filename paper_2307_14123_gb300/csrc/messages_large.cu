@@ -221,12 +221,13 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    // w'_{i, j0 + jj} of this lane's feature; zero past the block's senders (of an empty spin block
-    // not even slot 0 is one, and the pair table of the last receiver ends before it)
+    // w'_{i, j0 + jj} of this lane's feature; of an empty spin block (jn = 0, j0 may be N) some other
+    // sender's, whose product with za = 0 vanishes: past the row's end the pair table holds no edge
+    const int jw = min(j0, N - 1);
     auto w1_at = [&](int i, int jj) -> float {
       if (stage_w1) return W1[(i * NBS + jj) * 32 + lane];
-      const int j = j0 + jj;
-      return jj >= jn || i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
+      const int j = jw + jj;
+      return i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
     };
     // ---- the contraction: a warp task holds the 3 EPT coordinate channels of EPT consecutive
     // electrons (channel c = 1 + 3 e + x: electron e, axis x known per register slot), and one
