@@ -87,8 +87,10 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid) 
 
 // NBS: sender slots per spin block (at least the larger block); EPT: electrons per warp task (its
 // register tile is NBS x 3 EPT); NW: warps per CTA; SW1: the w' tables in shared memory (else read
-// from global memory where used).
-template <int NBS, int EPT, int NW, bool SW1, class TO>
+// from global memory where used); EMPTY: no spin-down electrons, whose pass has no senders.  A
+// parameter, because a test of the sender slot at every read of w' spills a register of the receiver
+// loop (benzene's messages, 250 walkers, two layers: 2.90 -> 3.12 ms).
+template <int NBS, int EPT, int NW, bool SW1, bool EMPTY, class TO>
 __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid_constant__ MLArgs a) {
   constexpr int CB = 3 * EPT;
   extern __shared__ __align__(16) float ml_smem[];
@@ -221,12 +223,10 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    // w'_{i, j0 + jj} of this lane's feature; of an empty spin block (jn = 0, j0 may be N) some other
-    // sender's, whose product with za = 0 vanishes: past the row's end the pair table holds no edge
-    const int jw = min(j0, N - 1);
-    auto w1_at = [&](int i, int jj) -> float {
+    auto w1_at = [&](int i, int jj) -> float {  // w'_{i, j0 + jj} of this lane's feature
       if (stage_w1) return W1[(i * NBS + jj) * 32 + lane];
-      const int j = jw + jj;
+      if (EMPTY && jj >= jn) return 0.f;  // not even slot 0 is a sender, and Ps may end before it
+      const int j = j0 + jj;
       return i == j ? 0.f : EWb[((int64_t)Ps[i * N + j] * 3 + 1) * D];
     };
     // ---- the contraction: a warp task holds the 3 EPT coordinate channels of EPT consecutive
@@ -391,7 +391,9 @@ __global__ void __launch_bounds__(NW * 32, 1) messages_large_kernel(const __grid
 template <int NBS, int EPT, int NW, class TO>
 cudaError_t launch_ml(const MLArgs& a, int64_t Bc, cudaStream_t s) {
   const MLSmem lay = ml_layout(a.N, NBS, a.stage_w1 != 0);
-  auto kern = a.stage_w1 ? messages_large_kernel<NBS, EPT, NW, true, TO> : messages_large_kernel<NBS, EPT, NW, false, TO>;
+  auto kern = a.stage_w1     ? messages_large_kernel<NBS, EPT, NW, true, false, TO>
+              : a.n_up < a.N ? messages_large_kernel<NBS, EPT, NW, false, false, TO>
+                             : messages_large_kernel<NBS, EPT, NW, false, true, TO>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total_bytes);
   if (e != cudaSuccess) return e;
   kern<<<dim3((unsigned)Bc, (unsigned)(a.D / kMLLanes)), NW * 32, lay.total_bytes, s>>>(a);
