@@ -805,8 +805,7 @@ cudaError_t launch_edge_update_bwd(const dq_handle_s& h, int64_t Bc, int l, cons
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = ((size_t)3 * Q * Q + 3 * Q + (size_t)3 * rpi * Q) * sizeof(T);
-  cudaError_t e = cudaFuncSetAttribute(edge_update_bwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(edge_update_bwd_kernel<T>, smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nblk, (int64_t)std::max(sms, 1) * 8));
   edge_update_bwd_kernel<T><<<grid, 256, smem, s>>>(fprev, ebar, abar, params, Bc, h.edges.n_all, h.edges.n_par,
@@ -841,7 +840,7 @@ cudaError_t launch_bwd_det(const dq_handle_s& h, int64_t Bc, const T* phi, const
   const int warps = 4;
   const size_t smem = per_warp * warps;
   auto kern = bwd_det_kernel<T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<nblocks(Bc * 2 * h.K, warps), warps * 32, smem, s>>>(
       phi, geo, params, beta, Bc, h.N, h.n_up, h.M, h.K, h.K * nmax, h.edges.n_all, h.edges.n_ee, h.off.omega[0],
@@ -1022,7 +1021,7 @@ cudaError_t launch_msg_bwd(const dq_handle_s& h, int64_t Bc, const T* mbar, cons
   const bool staged = slice <= kMbStage;
   const size_t smem = (staged ? slice : 0) + (size_t)h.N * 4 * 32 * sizeof(T) +
                       (size_t)(h.N * h.N + 2 * h.edges.n_ee) * sizeof(int);
-  cudaError_t e = cudaFuncSetAttribute(msg_bwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(msg_bwd_kernel<T>, smem);
   if (e != cudaSuccess) return e;
   msg_bwd_kernel<T><<<grid, 256, smem, s>>>(mbar, Z, z0, ew, Y, h.d_pair_ij, h.d_pair_of, h.N, h.n_up, h.M, h.D, h.edges.n_all,
                                           h.edges.n_ee, z_const ? 1 : 0, staged ? 1 : 0, zbar, wbar, ybar);

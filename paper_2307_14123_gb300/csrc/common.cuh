@@ -15,6 +15,20 @@ constexpr int kMaxSpin = 32;   // electrons per spin channel (one warp per matri
 constexpr int kMaxNuc = 64;
 constexpr size_t kMaxSmem = 232448;  // shared memory of a block, static arrays included (227 KB)
 
+// Lets launches of a kernel take `smem` bytes of dynamic shared memory.  The attribute is the
+// kernel's, not a launch's: set to the size of the call at hand, it could be lowered by another
+// thread's smaller call between this call's setting and its launch, which would then be refused.
+// So every call sets the same value, all but what is kept for the kernel's static arrays.
+inline cudaError_t allow_smem(const void* kern, size_t smem, size_t statics = 0) {
+  const size_t most = kMaxSmem - statics;
+  if (smem > most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+template <class... A>
+cudaError_t allow_smem(void (*kern)(A...), size_t smem, size_t statics = 0) {
+  return allow_smem(reinterpret_cast<const void*>(kern), smem, statics);
+}
+
 // Element offsets of the blocks of the flat parameter vector (layout in dqmc.h).
 struct ParamOffsets {
   int64_t E_spin;                    // -1 with the electron-nucleus initial embedding

@@ -2519,7 +2519,7 @@ cudaError_t launch_orbital_det(const dq_handle_s& h, const FwdDims& d, const T* 
   const int warps = per_warp * 4 <= 200 * 1024 ? 4 : 1;
   const size_t smem = per_warp * warps;
   auto kern = orbital_det_kernel<T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int64_t nmat = d.Bc * 2 * d.K;
   kern<<<blocks(nmat, warps), warps * 32, smem, s>>>(b.phi, b.geo, params, d.Bc, d.N, d.n_up, d.M, d.K, d.C,
@@ -2607,7 +2607,7 @@ cudaError_t launch_edge_hidden_group(const MolFwd<T>* m, int n, int l, cudaStrea
   // for 512 N2 walkers in FP32 at n_rbf 32, width 256, jets, two layers).
   int epb = kEdgesPerBlk;
   if (rows_all < (int64_t)4 * kEdgesPerBlk * device_sms() || smem_of(epb) > kMaxSmem) epb /= 2;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(epb));
+  cudaError_t e = allow_smem(kern, smem_of(epb));
   if (e != cudaSuccess) return e;
   if (epb == kEdgesPerBlk) {
     int occ = 0, occ_half = 0;
@@ -2656,8 +2656,7 @@ cudaError_t launch_edge_update_group(const MolFwd<T>* m, int n, int l, const T* 
           std::max<int64_t>(1, std::min<int64_t>(nblk, (int64_t)device_sms() * 8)));
   }
   if (g.n == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(edge_update_kernel_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(edge_update_kernel_group<T>, smem);
   if (e != cudaSuccess) return e;
   e = check_group(g);
   if (e != cudaSuccess) return e;
@@ -2673,7 +2672,7 @@ cudaError_t launch_el_init(const dq_handle_s& h, const FwdDims& d, const T* para
   int per = (int)std::min<size_t>(kElInitMax, (96 * 1024) / ((size_t)nch * D * sizeof(T) + M3 * sizeof(T)));
   per = std::max(per, 1);
   const size_t smem = (size_t)per * (M3 + nch * D) * sizeof(T);
-  cudaError_t e = cudaFuncSetAttribute(el_init_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(el_init_kernel<T>, smem);
   if (e != cudaSuccess) return e;
   const T* R = sizeof(T) == 8 ? reinterpret_cast<const T*>(h.d_R) : reinterpret_cast<const T*>(h.d_Rf);
   const int64_t n_el = d.Bc * h.N;
@@ -2729,8 +2728,7 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
             d.Bc, d.D / 32);
     }
     if (g.n == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(messages_value_kernel_group<T, TO>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(messages_value_kernel_group<T, TO>, smem);
     if (e != cudaSuccess) return e;
     e = check_group(g);
     if (e != cudaSuccess) return e;
@@ -2803,7 +2801,7 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
   }
   if (ne == 0) return cudaSuccess;
   auto kern = messages_kernel_group<T, TO, IB, CB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   // One launch per occupancy class: molecules whose CTAs fit the same number per SM share a
   // launch (the launch's shared memory is its largest entry's, which sets everyone's occupancy).
@@ -2910,7 +2908,7 @@ cudaError_t launch_orbital_det_group(const MolFwd<T>* m, int n, cudaStream_t s) 
   }
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < ne; ++i) {
-    e = cudaFuncSetAttribute(kerns[kind(ent[i].tag)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(kerns[kind(ent[i].tag)], smem);
     if (e != cudaSuccess) return e;
   }
   // one launch per kernel and occupancy class (see launch_messages_group)
@@ -2978,8 +2976,7 @@ cudaError_t launch_combine_group(const MolFwd<T>* m, int n, T* const* logabs, in
           d.Bc);
   }
   if (g.n == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(combine_kernel_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(combine_kernel_group<T>, smem, 1024);
   if (e != cudaSuccess) return e;
   combine_kernel_group<T><<<(unsigned)g.blocks(), kCombineThreads, smem, s>>>(g);
   return cudaGetLastError();

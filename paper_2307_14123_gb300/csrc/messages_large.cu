@@ -394,7 +394,7 @@ cudaError_t launch_ml(const MLArgs& a, int64_t Bc, cudaStream_t s) {
   auto kern = a.stage_w1     ? messages_large_kernel<NBS, EPT, NW, true, false, TO>
               : a.n_up < a.N ? messages_large_kernel<NBS, EPT, NW, false, false, TO>
                              : messages_large_kernel<NBS, EPT, NW, false, true, TO>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total_bytes);
+  cudaError_t e = allow_smem(kern, lay.total_bytes);
   if (e != cudaSuccess) return e;
   kern<<<dim3((unsigned)Bc, (unsigned)(a.D / kMLLanes)), NW * 32, lay.total_bytes, s>>>(a);
   return cudaGetLastError();

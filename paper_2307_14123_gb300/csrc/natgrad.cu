@@ -293,7 +293,7 @@ __global__ void ng_cg_direction_kernel(int64_t B, const double* __restrict__ z, 
 constexpr int kCgThreads = 512;
 constexpr int kCgWarps = kCgThreads / 32;
 constexpr int kCgMaxGroups = 64;                  // groups of kNgThreads walkers: B <= 16384
-constexpr size_t kCgMaxSmem = 227 * 1024 - 4096;  // 4 KB left for the static arrays
+constexpr size_t kCgStatics = 4096;               // kept for the static arrays
 
 inline size_t ng_solve_smem(int64_t B) { return (size_t)3 * B * sizeof(double); }
 
@@ -502,11 +502,11 @@ bool ng_solve(const double* T, int64_t B, const double* r, const double* p, cons
               CgScalars* sc, unsigned int* arrivals, unsigned int* status, cudaStream_t s, cudaError_t* e) {
   *e = cudaSuccess;
   const size_t smem = ng_solve_smem(B);
-  if (smem > kCgMaxSmem) return false;  // B > 9514
+  if (smem > kMaxSmem - kCgStatics) return false;  // B > 9514
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  *e = cudaFuncSetAttribute(ng_cg_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  *e = allow_smem(ng_cg_solve_kernel, smem, kCgStatics);
   if (*e == cudaSuccess)
     *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ng_cg_solve_kernel, kCgThreads, smem);
   if (*e != cudaSuccess) return true;
