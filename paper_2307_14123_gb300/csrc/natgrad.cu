@@ -27,7 +27,7 @@ constexpr int kNgRowWarps = 8;  // matvec: one warp per row of the Gram matrix
 // FP64 adds, multiply-adds and conversions from FP32 issue at 1.7 per clock and SM, 75 times slower
 // than FP32 ones: passes over G in FP64 were bound by them (one conversion, one operation per
 // element: 1.6 ms for 1024 x 412,656 gradients that memory delivers in 0.25 ms).  The sums below
-// (column means 1.62 -> 0.27 ms, centring 2.30 -> 0.48, the last product 1.60 -> 0.65)
+// (column means 1.62 -> 0.27 ms, centring 2.30 -> 0.59, the last product 1.60 -> 0.66)
 // are carried as three FP32 terms instead, hi + c1 + c2: every product and every addition into hi
 // and c1 keeps its rounding error exactly (TwoProd and TwoSum of Ogita, Rump, Oishi, "Accurate sum
 // and dot product", SIAM J. Sci. Comput. 26, 2005), so that only c2's additions round, at 2^-72 of
@@ -46,11 +46,18 @@ struct Sum3 {
   }
   __device__ __forceinline__ double value() const { return (double)hi + ((double)c1 + (double)c2); }
 };
+// x as the three FP32 terms whose sum it is
+__device__ __forceinline__ float4 split3(double x) {
+  const float h = (float)x;
+  const double r = x - (double)h;
+  const float l = (float)r;
+  return make_float4(h, l, (float)(r - (double)l), 0.f);
+}
 
-// mean[p] = (1 / B) sum_b G[b][p] as an FP32 pair (to 2^-48).  A CTA sums 32 columns, warp g the
-// rows g, g + 8, ..; the warps' sums are added in FP64.
+// mean[p] = (1 / B) sum_b G[b][p] in FP64, stored as the three FP32 terms that hold it exactly.  A
+// CTA sums 32 columns, warp g the rows g, g + 8, ..; the warps' sums are added in FP64.
 __global__ void __launch_bounds__(kNgThreads)
-    ng_colmean_kernel(const float* __restrict__ G, int64_t B, int64_t P, float2* __restrict__ mean) {
+    ng_colmean_kernel(const float* __restrict__ G, int64_t B, int64_t P, float4* __restrict__ mean) {
   __shared__ double sh[kNgThreads / 32][32];
   const int lane = threadIdx.x % 32, g = threadIdx.x / 32;
   const int64_t p = (int64_t)blockIdx.x * 32 + lane;
@@ -67,28 +74,46 @@ __global__ void __launch_bounds__(kNgThreads)
 #pragma unroll
     for (int k = 0; k < kNgThreads / 32; ++k) t += sh[k][lane];
     t /= (double)B;
-    const float h = (float)t;
-    mean[p] = make_float2(h, (float)(t - (double)h));
+    mean[p] = split3(t);
   }
 }
 
-// Gc[b][p] = G[b][p] - mean[p] (one rounding of the difference, up to 2^-20 of an ulp) with row
-// pitch Pp (zeros in the padding); a thread per column and 8 rows.
+// Gc[b][p] = G[b][p] - mean[p], the FP64 mean's three terms subtracted with one rounding, and row
+// pitch Pp (zeros in the padding); a thread per column and 8 rows.  g - mean is formed without error
+// as f.hi + f.lo + the rest, and the small parts are added with rounding to odd (the last bit tells
+// that more follows), so that f.hi + them rounds as the exact difference does (Boldo, Melquiond,
+// "Emulation of a FMA and correctly rounded sums: proved algorithms using rounding to odd", IEEE
+// Trans. Comput. 57, 2008).  The three terms and the odd roundings take 0.59 ms for 1024 x 412,656
+// gradients where two terms rounded as they come took 0.48, with up to 1.5 times the error.
 constexpr int kNgCenterRows = 8;
-__global__ void ng_center_kernel(const float* __restrict__ G, const float2* __restrict__ mean, int64_t B, int64_t P,
+__device__ __forceinline__ float add_odd(float a, float b) {  // a + b rounded to odd
+  const float d = __fadd_rd(a, b), u = __fadd_ru(a, b);  // of two neighbours one is odd
+  return (__float_as_int(d) & 1) ? d : u;
+}
+__device__ __forceinline__ float ng_minus_mean(float g, float4 m) {
+  const dfloat d = two_sum(g, -m.x);
+  const dfloat f = two_sum(d.hi, -m.y);
+  return __fadd_rn(f.hi, add_odd(f.lo, add_odd(d.lo, -m.z)));
+}
+__global__ void ng_center_kernel(const float* __restrict__ G, const float4* __restrict__ mean, int64_t B, int64_t P,
                                  int64_t Pp, float* __restrict__ Gc) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= Pp) return;
-  const float2 m = p < P ? mean[p] : make_float2(0.f, 0.f);
   const int64_t b0 = (int64_t)blockIdx.y * kNgCenterRows;
+  const int n = (int)min((int64_t)kNgCenterRows, B - b0);
+  float* out = Gc + b0 * Pp + p;
+  if (p >= P) {
+    for (int k = 0; k < n; ++k) out[k * Pp] = 0.f;
+    return;
+  }
+  const float4 m = mean[p];
+  const float* in = G + b0 * P + p;
   float g[kNgCenterRows];
 #pragma unroll
-  for (int k = 0; k < kNgCenterRows; ++k) g[k] = p < P && b0 + k < B ? __ldg(G + (b0 + k) * P + p) : 0.f;
+  for (int k = 0; k < kNgCenterRows; ++k) g[k] = k < n ? __ldg(in + k * P) : 0.f;
 #pragma unroll
-  for (int k = 0; k < kNgCenterRows; ++k) {
-    const dfloat d = two_sum(g[k], -m.x);
-    if (b0 + k < B) Gc[(b0 + k) * Pp + p] = __fadd_rn(d.hi, __fsub_rn(d.lo, m.y));
-  }
+  for (int k = 0; k < kNgCenterRows; ++k)
+    if (k < n) out[k * Pp] = ng_minus_mean(g[k], m);
 }
 
 struct CgScalars {
@@ -447,11 +472,7 @@ __global__ void __launch_bounds__(kCgThreads, 1)
 // x as three FP32 terms (exact): the coefficients of ng_apply_kernel
 __global__ void ng_split_x_kernel(const double* __restrict__ x, int64_t B, float4* __restrict__ x3) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const float h = (float)x[b];
-  const double r1 = x[b] - (double)h;
-  const float l = (float)r1;
-  x3[b] = make_float4(h, l, (float)(r1 - (double)l), 0.f);
+  if (b < B) x3[b] = split3(x[b]);
 }
 
 // delta[p] = sum_b x_b Gc[b][p] (fixed order): a CTA 32 columns, warp g the rows g, g + 8, ..
@@ -528,7 +549,7 @@ size_t natgrad_workspace(int64_t B, int64_t P) {
   const int64_t Pp = (P + 3) / 4 * 4;
   const int64_t mv_ctas = (B + kNgRowWarps - 1) / kNgRowWarps;
   size_t o = 0;
-  o += ng_align((size_t)P * 8);                 // mean
+  o += ng_align((size_t)P * 16);                // mean in three FP32 terms
   o += ng_align((size_t)B * Pp * 4);            // Gc
   o += ng_align((size_t)kNgJobs * B * B * 4);  // Gram matrices of the chunks of one launch
   o += ng_align((size_t)B * B * 8);             // Gram matrix (FP64)
@@ -551,7 +572,7 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
     o += ng_align(bytes);
     return q;
   };
-  float2* mean = reinterpret_cast<float2*>(take((size_t)P * 8));
+  float4* mean = reinterpret_cast<float4*>(take((size_t)P * 16));
   float* Gc = reinterpret_cast<float*>(take((size_t)B * Pp * 4));
   float* Tc = reinterpret_cast<float*>(take((size_t)kNgJobs * B * B * 4));
   double* T = reinterpret_cast<double*>(take((size_t)B * B * 8));
