@@ -10,6 +10,7 @@
 // Gc^T x is a weighted column sum.  The conjugate gradients run in one cooperative kernel whose
 // CTAs meet at one grid barrier per iteration and leave the loop when the residual is small
 // enough, so the call needs no host synchronisation and can be captured in a CUDA graph.
+#include <float.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -67,7 +68,12 @@ __global__ void __launch_bounds__(kNgThreads)
 #pragma unroll 8
     for (int64_t b = g; b < B; b += kNgThreads / 32) s.add(__ldg(q + b * P));
   }
-  sh[g][lane] = s.value();
+  double v = s.value();
+  if (!(fabsf(s.hi + (s.c1 + s.c2)) <= FLT_MAX)) {  // a sum past FP32's range (or not a number): in FP64
+    v = 0;
+    for (int64_t b = g; b < B; b += kNgThreads / 32) v += (double)__ldg(G + b * P + p);
+  }
+  sh[g][lane] = v;
   __syncthreads();
   if (g == 0 && p < P) {
     double t = 0;
@@ -119,6 +125,7 @@ __global__ void ng_center_kernel(const float* __restrict__ G, const float4* __re
 struct CgScalars {
   double rr, rr0, rz, pAp, beta, lam;
   double tol2;  // (tol ||w||)^2
+  double xback;  // 1 / the scale of x in three FP32 terms
   int iter, max_iter, done, pad;
   unsigned int counter;  // arrivals of the CTAs of the current reduction
 };
@@ -469,16 +476,32 @@ __global__ void __launch_bounds__(kCgThreads, 1)
   }
 }
 
-// x as three FP32 terms (exact): the coefficients of ng_apply_kernel
-__global__ void ng_split_x_kernel(const double* __restrict__ x, int64_t B, float4* __restrict__ x3) {
+// The coefficients of ng_apply_kernel: x as three FP32 terms, scaled by the power of two that takes
+// the largest |x| to 2^40: its products with FP32 gradients then neither overflow (gradients past 2^64
+// already overflow the Gram matrix's FP32 sums) nor lose their rounding errors to underflow, whatever
+// the size of x.  Every CTA finds the largest exponent by itself.
+constexpr int kNgScaleExp = 40;
+__global__ void __launch_bounds__(kNgThreads)
+    ng_split_x_kernel(const double* __restrict__ x, int64_t B, CgScalars* sc, float4* __restrict__ x3) {
+  __shared__ int s_e;
+  if (threadIdx.x == 0) s_e = 0;
+  __syncthreads();
+  int e = 0;
+  for (int64_t i = threadIdx.x; i < B; i += blockDim.x) e = max(e, (__double2hiint(x[i]) >> 20) & 0x7ff);
+  atomicMax(&s_e, e);
+  __syncthreads();
+  e = max(s_e, kNgScaleExp + 1);              // biased exponent (clamped: the scale stays below 2^1023)
+  if (e == 0x7ff) e = 1023 + kNgScaleExp;     // not finite: no scale
+  const double up = __hiloint2double((2 * 1023 + kNgScaleExp - e) << 20, 0);
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) x3[b] = split3(x[b]);
+  if (b < B) x3[b] = split3(x[b] * up);
+  if (b == 0) sc->xback = __hiloint2double((e - kNgScaleExp) << 20, 0);
 }
 
 // delta[p] = sum_b x_b Gc[b][p] (fixed order): a CTA 32 columns, warp g the rows g, g + 8, ..
 __global__ void __launch_bounds__(kNgThreads)
     ng_apply_kernel(const float* __restrict__ Gc, int64_t B, int64_t P, int64_t Pp, const float4* __restrict__ x3,
-                    float* __restrict__ delta) {
+                    const CgScalars* __restrict__ sc, float* __restrict__ delta) {
   __shared__ double sh[kNgThreads / 32][32];
   const int lane = threadIdx.x % 32, g = threadIdx.x / 32;
   const int64_t q = (int64_t)blockIdx.x * 32 + lane;
@@ -503,7 +526,7 @@ __global__ void __launch_bounds__(kNgThreads)
     double t = 0;
 #pragma unroll
     for (int k = 0; k < kNgThreads / 32; ++k) t += sh[k][lane];
-    delta[q] = (float)t;
+    delta[q] = (float)(t * sc->xback);
   }
 }
 
@@ -643,8 +666,8 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
     }
   }
   if (e != cudaSuccess) return e;
-  ng_split_x_kernel<<<ng_blocks(B, kNgThreads), kNgThreads, 0, s>>>(x, B, x3);
-  ng_apply_kernel<<<ng_blocks(P, 32), kNgThreads, 0, s>>>(Gc, B, P, Pp, x3, delta);
+  ng_split_x_kernel<<<ng_blocks(B, kNgThreads), kNgThreads, 0, s>>>(x, B, sc, x3);
+  ng_apply_kernel<<<ng_blocks(P, 32), kNgThreads, 0, s>>>(Gc, B, P, Pp, x3, sc, delta);
   if (stats) ng_stats_kernel<<<1, 1, 0, s>>>(sc, stats);
   return cudaGetLastError();
 }
