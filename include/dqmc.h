@@ -497,8 +497,10 @@ dq_status dq_msg_tile(dq_handle h, int32_t* msg_ib);
  * their node channels for up to 11 channels in registers and runs over every
  * receiver; FP32 and BF16 modes, width a multiple of 32, at most 48
  * electrons, 24 per spin); mode 0 (the default) is mode 2 above 16 electrons
- * where supported and mode 1 elsewhere.  Layers whose node channels are the
- * spin-embedding constants always take the general kernel.  Mode 2 on a DQ_FP64
+ * where supported and the general kernel elsewhere.  In modes 0 and 2, layers
+ * of FP32 and BF16 handles whose node channels are the spin-embedding constants
+ * take a kernel of their own with the general kernel's bits; in mode 1 they take
+ * the general kernel too.  Mode 2 on a DQ_FP64
  * handle: DQ_ERR_UNSUPPORTED; other modes: DQ_ERR_ARG.  Both kernels compute
  * the same messages within FP32 rounding (different summation orders).
  * dq_msg_kernel reports the kernel the handle's jet layers take on the

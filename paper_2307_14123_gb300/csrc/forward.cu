@@ -2749,8 +2749,8 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
     if (d.Bc <= 0) continue;
     if (d.D % kMsgLanes) return cudaErrorInvalidConfiguration;
     if constexpr (sizeof(T) == 4) {
-      // constant node channels: a kernel of their own
-      if (z_const && !h.el_init) {
+      // constant node channels: a kernel of their own (unless the handle asks for the general one)
+      if (z_const && !h.el_init && h.msg_kernel != 1) {
         cudaError_t e = launch_messages_const(h, d, reinterpret_cast<const float*>(m[k].params), l,
                                               reinterpret_cast<const float*>(m[k].b.z0),
                                               reinterpret_cast<const float*>(m[k].b.ew),
