@@ -539,7 +539,7 @@ dq_status dq_tile_set(dq_handle h, int64_t* max_chunk, int32_t* msg_ib, int32_t*
  *                                      buffer),
  *   walker chunk   4096, 2048        (dq_set_max_chunk: the M extent of every
  *                                      GEMM, the grid of every other kernel),
- *   msg_ib         8, 4              (separate message kernel only),
+ *   msg_ib         8, 4              (where the general message kernel runs),
  *   det warps      4, 2              (dq_set_det_warps; with the 4096 chunk),
  * one warm-up and two timed calls each (CUDA events on `stream`, host waits),
  * and keeps the fastest; workspace: at least dq_workspace_size(op =

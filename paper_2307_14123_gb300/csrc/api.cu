@@ -2096,6 +2096,17 @@ TuneKey tune_key(const dq_handle_s& h, int64_t B) {
 }
 }  // namespace
 
+namespace {
+// Whether some launch of the separate layer path reads msg_ib: the general message kernel, which
+// serves layers with mapped node channels where the sender-tiled kernel does not.
+bool reads_msg_tile(const dq_handle_s& h) {
+  if (h.msg_kernel == 1) return true;
+  const FwdDims d{1, h.N, h.n_up, h.n_dn, h.M, h.D, h.K, h.Q, 3 * h.N + 2};
+  const bool tiled = (h.msg_kernel == 2 || h.N > 16) && messages_large_supported(h, d);
+  return !tiled && (h.L > 1 || h.el_init);
+}
+}  // namespace
+
 dq_status dq_autotune(dq_handle h, const void* params, const void* r, int64_t B, void* ws, size_t ws_bytes,
                       void* stream, double* best_ms) {
   dq_status st = check_handle(h);
@@ -2155,7 +2166,7 @@ dq_status dq_autotune(dq_handle h, const void* params, const void* r, int64_t B,
       // kernels' CTA size is tried with the largest chunk only
       for (int cand = 0; cand < 3; ++cand) {
         const int ib = cand == 1 ? 4 : 8, dw = cand == 2 ? 2 : 4;
-        if ((lk == 1 && cand == 1) || (cand == 2 && chunk != 4096)) continue;
+        if ((cand == 1 && (lk == 1 || !reads_msg_tile(*h))) || (cand == 2 && chunk != 4096)) continue;
         h->layer_kernel = lk;
         h->max_chunk = chunk;
         h->msg_ib = ib;
@@ -2232,10 +2243,13 @@ dq_status dq_autotune_multi(dq_multi g, const void* const* params, const void* c
   double best = -1;
   int best_rounds = keep_rounds, best_ib = keep_ib;
   st = DQ_OK;
+  bool tile = false;  // some molecule's launches read msg_ib
+  for (int m = 0; m < g->n; ++m) tile = tile || (!use_fused(*g->h[m], true) && reads_msg_tile(*g->h[m]));
   for (int rounds = 1; rounds <= 4 && st == DQ_OK; ++rounds) {
     g->rounds = rounds;
     if (plan_forward_multi(*g, B, true, 4).total > fwd_bytes) continue;
     for (int ib : {8, 4}) {
+      if (ib == 4 && !tile) continue;
       for (int m = 0; m < g->n; ++m) g->h[m]->msg_ib = ib;
       float ms = 0;
       for (int rep = 0; rep < 3 && st == DQ_OK; ++rep) {
