@@ -138,8 +138,13 @@ struct Vec16<double> {
   static constexpr int n = 2;
 };
 
-// Edges per block: 32, or 16 where 32 would leave an SM fewer than four blocks (a count of blocks
-// per SM that rounds up costs less then) or would not fit (launch_edge_hidden_group).
+// Edges per block: 32, or 16 where 32 would not fit (launch_edge_hidden_group) or would load the SMs
+// too unevenly.  FP32: fewer than one block of 32 per SM (three layers, values / jets: 20 N2 walkers,
+// 2380 edges, 18.9 / 22.5 us with 16, 23.5 / 28.7 with 32; from there on the better use of a W1 load
+// counts: 77 walkers 35.1 / 61.8 against 28.8 / 49.2, 20 C4H4 walkers 80.7 / 112 against 55.8 / 95.5).
+// FP64, bound by the FP64 pipe of the busiest SM: fewer than four blocks per SM (100 LiH walkers 34 /
+// 50 us with 16, 50 / 81 with 32; 700: 94 / 176 and 112 / 211; 1200: 140 / 246 and 146 / 277; 1389,
+// 19,446 edges: 170 / 281 and 148 / 280; 2000: 206 / 399 either way).
 constexpr int kEdgesPerBlk = 32;
 constexpr int kHiddenThreads = 256;
 
@@ -2606,7 +2611,8 @@ cudaError_t launch_edge_hidden_group(const MolFwd<T>* m, int n, int l, cudaStrea
   // two: 1886 us against 1208 for 2048 LiH walkers in FP64 at n_rbf 32, width 96; 384 against 322
   // for 512 N2 walkers in FP32 at n_rbf 32, width 256, jets, two layers).
   int epb = kEdgesPerBlk;
-  if (rows_all < (int64_t)4 * kEdgesPerBlk * device_sms() || smem_of(epb) > kMaxSmem) epb /= 2;
+  const int64_t few = (sizeof(T) == 8 ? 4 : 1) * (int64_t)kEdgesPerBlk * device_sms();
+  if (rows_all < few || smem_of(epb) > kMaxSmem) epb /= 2;
   cudaError_t e = allow_smem(kern, smem_of(epb));
   if (e != cudaSuccess) return e;
   if (epb == kEdgesPerBlk) {
