@@ -635,10 +635,14 @@ __global__ void add_rows_kernel(T* __restrict__ fbar, const T* __restrict__ sbar
 // The kernel is bound by the latency of its reads, so everything that is used
 // more than once is staged in shared memory first: z, the message adjoints, and
 // the CTA's slice of the filters (16-byte loads, all issued before any is used;
-// slices above kMbStage bytes are read in place): three layers of 4096 N2 walkers
-// 1.03 -> 0.64 ms.
+// slices above kMbStage bytes and of fewer than kMbStageMin edges are read in
+// place): three layers of 4096 N2 walkers 1.03 -> 0.64 ms.  Staged / read in place,
+// width 128, 4096 walkers of 14 edges 173 / 149 us, of 75 edges (9 KB) 439 / 461; 2048 of 216
+// (27 KB) 497 / 485 and 200 of them at width 64 41 / 53; 1024 of 324 (41 KB) 503 / 403, of 420
+// 598 / 465.  FP64, width 64, 512 walkers of 119 edges (30 KB) 150 / 185, of 184 (46 KB) 260 / 225.
 // ---------------------------------------------------------------------------
-constexpr size_t kMbStage = 64 * 1024;
+constexpr size_t kMbStage = 32 * 1024;
+constexpr int kMbStageMin = 32;
 template <class T>
 __global__ void __launch_bounds__(256)
     msg_bwd_kernel(const T* __restrict__ mbar, const T* __restrict__ Z, const T* __restrict__ z0,
@@ -1018,7 +1022,7 @@ cudaError_t launch_msg_bwd(const dq_handle_s& h, int64_t Bc, const T* mbar, cons
   if (h.D % 32) return cudaErrorInvalidValue;
   dim3 grid((unsigned)Bc, h.D / 32);
   const size_t slice = (size_t)h.edges.n_all * 32 * sizeof(T);
-  const bool staged = slice <= kMbStage;
+  const bool staged = slice <= kMbStage && h.edges.n_all >= kMbStageMin;
   const size_t smem = (staged ? slice : 0) + (size_t)h.N * 4 * 32 * sizeof(T) +
                       (size_t)(h.N * h.N + 2 * h.edges.n_ee) * sizeof(int);
   cudaError_t e = allow_smem(msg_bwd_kernel<T>, smem);

@@ -924,17 +924,18 @@ __global__ void __launch_bounds__(256, 2) messages_kernel_group(const __grid_con
 // any is used): reading the filters where they are multiplied, twice per pair
 // and four at a time, was bound by latency: three layers of 4096 N2 walkers
 // 0.48 -> 0.35 ms.
-// Slices above kMvStage bytes (about 500 edges) are read in place: they would
-// leave too few CTAs per SM.
-constexpr size_t kMvStage = 64 * 1024;
+// Between kMvStageMin and kMvStageMax edges: with few a CTA waits for its copies
+// longer than for its reads, with many the copies crowd the CTAs out of an SM and the
+// reads overlap by themselves.  Three layers of width 128, staged / read in place: 4096 walkers of 14
+// edges 101 / 83 us, of 75 edges 261 / 272, of 119 342 / 364; 2048 of 152 edges 208 / 191, of 216
+// 271 / 224; 1024 of 420 edges 304 / 216.  FP64, width 64, 512 walkers: 75 edges 94 / 104, 119 126 / 129,
+// 184 152 / 155, 216 184 / 165.
+constexpr int kMvStageMin = 32, kMvStageMax = 128;
 template <class T>
 inline size_t mv_tables(int N) {  // z and the pair table, padded to the filters' 16 bytes
   return ((size_t)N * 32 * sizeof(T) + (size_t)N * N * sizeof(int) + 15) / 16 * 16;
 }
-template <class T>
-inline bool mv_staged(int E) {
-  return (size_t)E * 32 * sizeof(T) <= kMvStage;
-}
+inline bool mv_staged(int E) { return E >= kMvStageMin && E <= kMvStageMax; }
 template <class T, class TO>
 struct messages_value_kernel_args {
   const T* Z;
@@ -2727,7 +2728,7 @@ cudaError_t launch_messages_group_t(const MolFwd<T>* m, int n, int l, bool z_con
       const FwdDims& d = m[k].d;
       if (d.Bc <= 0) continue;
       if (d.D % 32) return cudaErrorInvalidConfiguration;
-      const bool staged = mv_staged<T>(h.edges.n_all);
+      const bool staged = mv_staged(h.edges.n_all);
       smem = std::max(smem, mv_tables<T>(d.N) + (staged ? (size_t)h.edges.n_all * 32 * sizeof(T) : 0));
       g.add({m[k].b.Z, m[k].b.z0, m[k].b.ew, m[k].params + h.off.layer[l].Y, h.d_pair_of, d.Bc, d.N, d.n_up, d.M, d.D,
              h.edges.n_all, h.edges.n_ee, z_const && !h.el_init ? 1 : 0, out_of(m[k]), staged ? 1 : 0},
