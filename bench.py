@@ -411,7 +411,7 @@ def roofline_for(kind, ms, n, wl, chunk, pk, how, alu, steps):
         flops = message_flops_per_walker(wl) * chunk
         peak = alu["fp32_tflops"] if wl.precision != "fp64" else alu["fp64_tflops"]
         ach = flops / t / 1e12
-        byts = (chunk * N * C * D * el * (L - 1) / L) + chunk * E * 3 * D * el + chunk * N * (2 * C + 15 if N >= 9 else 3 * C) * D * (2 if bf16 else el)
+        byts = (chunk * N * C * D * el * (L - 1) / L) + chunk * E * 3 * D * el + chunk * N * (2 * C + 15 if N >= (17 if bf16 else 9) else 3 * C) * D * (2 if bf16 else el)
         traffic = None
         if wl.name == "n2_fp32" and MSG_DRAM_BYTES_PER_WALKER:
             traffic = MSG_DRAM_BYTES_PER_WALKER * chunk

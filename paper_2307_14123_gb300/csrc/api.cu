@@ -344,7 +344,7 @@ dq_status run_forward(const dq_handle_s& h, const T* params, const T* r, int64_t
   for (int64_t b0 = 0; b0 < B; b0 += Bmax) {
     const int64_t nb = std::min<int64_t>(Bmax, B - b0);
     const FwdDims d{nb, N, h.n_up, h.n_dn, h.M, D, K, h.Q, C};
-    place_split(bf, d, split_messages(d) && !use_fused(h, jets));
+    place_split(bf, d, split_messages(d, use_tc) && !use_fused(h, jets));
     DQ_LAUNCH(h, kb + PK_GEOMETRY, launch_geometry<T>(h, d, r + b0 * N * 3, bf, s));
     // embeddings of the electron-nucleus difference vectors (Eq. 13, second case): layer 0 then
     // takes the general path below instead of the spin-embedding shortcut
@@ -1091,7 +1091,7 @@ dq_status run_forward_multi(const dq_multi_s& g, const T* const* params, const T
         rest[m] = mf[m];
         fused[m] = use_fused(*g.h[m], jets) && mf[m].d.Bc > 0;
         if (fused[m]) rest[m].d.Bc = 0;
-        place_split(rest[m].b, rest[m].d, split_messages(rest[m].d) && rest[m].d.Bc > 0);
+        place_split(rest[m].b, rest[m].d, split_messages(rest[m].d, use_tc) && rest[m].d.Bc > 0);
       }
       DQ_LAUNCH(H, kb + PK_MESSAGES, launch_messages_group<T>(rest, n, l, l == 0, s));
       nj = 0;

@@ -327,8 +327,13 @@ struct FwdBuffers {
 };
 // Where the split pays: the update map reads 2 C + 15 instead of 3 C blocks per electron, for two
 // more launches.  C = 3 N + 2 >= 29 saves 15 % and more of the map and of the message traffic; both
-// parts fit the unsplit buffer from C = 25 on.
-inline bool split_messages(const FwdDims& d) { return d.C > 1 && d.N >= 9; }
+// parts fit the unsplit buffer from C = 25 on.  FP32 and FP64 from 9 electrons (local energies, three
+// layers, unsplit / split: 2048 walkers of 9 electrons at width 256 10.64 / 10.36 ms, of 10 12.42 /
+// 11.89; FP64, 1024 of 9 at width 32 8.86 / 8.27; 300 of 9 at width 64 845 / 826 us).  BF16 operands
+// are half the bytes and their map is not bound by them: there from 17 electrons, the sender-tiled
+// kernel's, whose stores they also save (width 256: 1024 of 10 5.36 / 5.48 ms, of 16 12.29 / 12.58; 512 of
+// 20 7.80 / 7.62, of 28 13.86 / 13.50).
+inline bool split_messages(const FwdDims& d, bool bf16) { return d.C > 1 && d.N >= (bf16 ? 17 : 9); }
 // Places a chunk's split messages in the buffers of the unsplit ones.
 template <class T>
 void place_split(FwdBuffers<T>& b, const FwdDims& d, bool split) {
