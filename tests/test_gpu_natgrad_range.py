@@ -70,3 +70,60 @@ def test_solutions_outside_fp32(g_exp, w_exp):
     normal = want.abs() >= 2.0 ** -126  # (below, FP32 results have fewer bits)
     assert float(normal.double().mean()) > 0.5
     assert torch.equal(d.double()[normal], want[normal])
+
+
+def _tiles(n, tri):
+    """Output tiles of an n x n Gram matrix: 256 x 128, all or those that reach row >= column."""
+    mp, nt = -(-n // 256), -(-n // 128)
+    return mp * (mp - 1) + min(2 * mp, nt) if tri else mp * nt
+
+
+def _waves(n, chunks, tri):
+    """Fewest waves of tiles over the chunks per launch (1 to 16), and that number of chunks."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return min((chunks // j * -(-j * _tiles(n, tri) // sms) + -(-(chunks % j) * _tiles(n, tri) // sms), -j)
+               for j in range(1, 17))
+
+
+def _solve64(G, w, lam):
+    Gc = G.double() - G.double().mean(dim=0)
+    T = Gc @ Gc.t() / G.shape[0]
+    T.diagonal().add_(lam)
+    return torch.linalg.solve(T, w.double()) @ Gc
+
+
+def _synthetic(B, P, seed):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    G = torch.randn(B, P, device=DEV, generator=g) * (0.05 + 1.95 * torch.rand(P, device=DEV, generator=g))
+    G += torch.randn(P, device=DEV, generator=g)
+    w = torch.randn(B, device=DEV, generator=g)
+    return G, (2.0 / B) * (w - w.mean())
+
+
+def test_triangular_gram_over_several_launches():
+    """600 walkers x 400,000 parameters: the half of the Gram matrix that is computed saves waves, its
+    chunks take several launches, and the last row and column blocks are ragged.  Against a dense FP64
+    solution, with the bound of the other parity tests (condition below 1e3)."""
+    h, B = _handle("n2_fp32"), 600
+    chunks = -(-h.P // 8192)
+    (full, _), (half, j) = _waves(B, chunks, False), _waves(B, chunks, True)
+    assert half < full and chunks > 2 * -j
+    G, w = _synthetic(B, h.P, 1)
+    lam = 0.1 * float(G.double().var(dim=0, unbiased=False).sum()) / B
+    d, st = h.natural_gradient(G, w, lam, max_iter=400, tol=1e-9)
+    ref = _solve64(G, w, lam)
+    assert float(st[1]) <= 1e-9 and float((d.double() - ref).norm()) <= 2e-3 * float(ref.norm())
+
+
+@pytest.mark.parametrize("B", [9514, 9515])
+def test_largest_one_kernel_solve_and_the_loop(B):
+    """The largest system of the one-kernel solve and the smallest of the launches per iteration,
+    against a dense FP64 solution (condition below 1e3: the largest eigenvalue of the random matrix is
+    about four times the mean)."""
+    from paper_2307_14123_gb300 import Ansatz
+    h = Ansatz(fx.molecule("H"), fx.AnsatzCfg(32, 1, 1), "fp32", device=DEV)
+    G, w = _synthetic(B, h.P, 2)
+    d, st = h.natural_gradient(G, w, -0.1, max_iter=400, tol=1e-9)
+    ref = _solve64(G, w, float(st[3]))
+    assert 1 <= float(st[0]) < 400 and float(st[1]) <= 1e-9
+    assert float((d.double() - ref).norm()) <= 2e-3 * float(ref.norm())
