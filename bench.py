@@ -297,7 +297,7 @@ MSG_DRAM_BYTES_PER_WALKER = None
 LAYER_FUSED_DRAM_BYTES_PER_WALKER = (234.25e6 + 108.18e6) / 512
 # the same for one launch of the sender-tiled message kernel (layer 1 of C4H4 in BF16 mode, 256
 # walkers; summary under profiles/); None once the kernel has changed since that capture.
-MSG_LARGE_DRAM_BYTES_PER_WALKER = None
+MSG_LARGE_DRAM_BYTES_PER_WALKER = (1.409136e9 + 0.746382e9) / 256
 
 
 def gemm_shapes(wl, chunk):

@@ -292,7 +292,7 @@ dq_status grad_logpsi(dq_handle h, const void* params, const void* r, int64_t B,
  * Gc Gc^T is formed on the tensor cores (3 x TF32 products); the system is
  * solved in FP64 with fixed-order reductions (deterministic).  FP32 and BF16
  * handles (DQ_ERR_UNSUPPORTED in FP64 mode); B >= 2.  Workspace:
- * dq_workspace_size(op = DQ_OP_NATGRAD, B), about 12 B P bytes. */
+ * dq_workspace_size(op = DQ_OP_NATGRAD, B), about 4 B P + 72 B^2 bytes. */
 dq_status natural_gradient(dq_handle h, const void* G, const void* w, int64_t B, double lambda, int32_t max_iter,
                            double tol, void* delta, double* stats, void* ws, size_t ws_bytes, void* stream);
 

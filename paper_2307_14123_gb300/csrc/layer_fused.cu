@@ -1,20 +1,20 @@
-// One graph-convolution layer of the jets forward pass in one kernel (FP32
-// and BF16 modes): the messages of Eq. 17 with their product-rule Jacobian and
-// Laplacian channels, the update map W_g of Eq. 18 on the tensor cores, and
-// the residual tanh update with its jet,
-//   f <- f + tanh(u),  J(tanh u) = t' J(u),  L(tanh u) = t' L(u) + t'' sum_k J_k(u)^2,
-//   u = W_g [m_par; m_anti; m_nuc] + b_g.
-// The messages are the A operand of the MMAs and never leave the SM; the
-// pre-activations u stay in tensor memory until the epilogue applies the
-// update to f in place.  Per walker the kernel reads the node map z (written
-// by the node-map GEMM), the filter jets, the geometry and f, and writes f.
+// The electron-electron part of a graph-convolution layer of the jets forward pass in one
+// kernel (FP32 and BF16 modes): the messages of Eq. 17 with their product-rule Jacobian
+// and Laplacian channels and their two blocks of the update map W_g of Eq. 18 on the
+// tensor cores, U = W_g [m_par; m_anti].
+// The messages are the A operand of the MMAs and never leave the SM.  Per walker the
+// kernel reads the node map z (written by the node-map GEMM), the filter jets and the
+// geometry, and writes U over z.  The electron-nucleus part W_g m_nuc + b_g, non-zero on
+// five channels per electron, is formed by a small GEMM and added by the kernel that
+// follows; the update kernel then applies
+//   f <- f + tanh(u),  J(tanh u) = t' J(u),  L(tanh u) = t' L(u) + t'' sum_k J_k(u)^2.
 //
 // Rows of a tile: one walker, the three coordinate channels of EPT consecutive
 // electrons (128 / N channels at most; the last tile takes the Laplacian and the
 // value channel too) and all N receivers i, row = (channel's place) N + i.  One
 // CTA processes a walker's tiles in electron order, the Laplacian last, so that
-// its cross terms accumulate on chip.  K steps: for each edge type t (same spin, opposite spin, nucleus)
-// and 32-feature block, A[row][32] = m_i^t[c][32 features] as three TF32
+// its cross terms accumulate on chip.  K steps: for each 32-feature block and edge type t (same
+// spin, opposite spin), A[row][32] = m_i^t[c][32 features] as three TF32
 // products with the W_g block (hi hi + hi lo + lo hi), or in BF16 mode as
 // one product of BF16 operands (FP32 accumulation).
 //
@@ -63,7 +63,7 @@ constexpr int LF_D = 128;                  // embedding width (the MMA's N)
 constexpr int LF_NFB = LF_D / LF_BK;       // feature blocks per edge type
 constexpr int LF_KSTEPS = 2 * LF_NFB;      // K = 2 D: the electron-electron blocks of W_g
 constexpr int LF_STAGES = 2;
-constexpr int LF_PROD = 16;                // producer warps at most (one per receiver)
+constexpr int LF_PROD = 16;                // receivers at most (a geometry table each)
 constexpr int LF_PROD_WARPS = 8;
 constexpr int LF_PROD_WARP0 = 6;           // warps 0 TMA, 1 MMA, 2-5 epilogue, 6-13 producers
 constexpr int LF_THREADS = (LF_PROD_WARP0 + LF_PROD_WARPS) * 32;

@@ -314,7 +314,8 @@ __global__ void ng_cg_direction_kernel(int64_t B, const double* __restrict__ z, 
 // CTA does.  That spends 6 B redundant multiply-adds per CTA instead of a second
 // barrier with its reduction, and every CTA takes the same decisions from the
 // same bits.  The sums are added in the order of the kernels above, which serve
-// the systems that do not fit here: both give the same bits.
+// the systems that do not fit here, with their roundings: with either form forced,
+// systems of 2 to 2000 walkers gave the same solutions and iteration counts bit for bit.
 // Against those (three launches per iteration, always max_iter of them; 17.4 +
 // 9.9 + 3.1 us each at B = 1024 until the residual is small) the call on 1024
 // walkers x 412,656 parameters took 15.2 ms instead of 17.7, and a LiH training
@@ -623,6 +624,9 @@ cudaError_t natgrad_run(const float* G, const float* w, int64_t B, int64_t P, do
   // launches of 16 chunks, 7 as triangles in launches of 15.  The triangle is taken where it saves
   // a wave; where it does not (a few chunks fill one wave either way) both halves are computed and
   // averaged.  (5.3 ms of launches with W split in memory first, 1.2 ms more, are 2.8 ms so.)
+  // The triangle costs no accuracy: T_ij and T_ji carry the same error of the FP32 sums, so that their
+  // average does not reduce it (largest and rms errors against 64 bits equal to four digits for N2, LiH
+  // and H2O gradients and random ones; N2, 1024 walkers: 7.16e-5 and 4.70e-5 of sqrt(T_ii T_jj)).
   const int64_t n_chunks = (Pp + kNgChunk - 1) / kNgChunk;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
